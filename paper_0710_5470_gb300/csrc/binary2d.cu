@@ -475,23 +475,30 @@ __global__ void binary_init_kernel(const double* rho, const double* phi, const d
 
 // Observables in float64: rho, phi, u (Eq. 3) and mu; in the forcing scheme
 // also M'_xx - M'_yy and M'_xy for binary_velocity_kernel.
-template <class real>
+// Bound by the FP64 pipe: conversions in integer instructions (lbk::widen) and
+// the momentum, its divisions and u only with WANT_U.
+template <class real, bool WANT_U>
 __global__ void binary_moments_kernel(const real* src, long long pitch, int nx, int ny, double* rho, double* phi,
                                       double* ux, double* uy) {
     const long long n = (long long)nx * ny;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         double r = 0, p = 0, jx = 0, jy = 0;
-        for (int i = 0; i < Q; ++i) {
-            const double fi = double(src[i * pitch + s]);
+        static_for<0, Q>([&](auto K) {
+            constexpr int i = decltype(K)::value;
+            const double fi = lbk::widen(src[i * pitch + s]);
             r += fi;
-            jx += D2Q9::ex(i) * fi;
-            jy += D2Q9::ey(i) * fi;
-            p += double(src[(Q + i) * pitch + s]);
-        }
+            p += lbk::widen(src[(Q + i) * pitch + s]);
+            if constexpr (WANT_U) {
+                jx = signed_add<D2Q9::ex(i)>(jx, fi);
+                jy = signed_add<D2Q9::ey(i)>(jy, fi);
+            }
+        });
         rho[s] = r;
         phi[s] = p;
-        ux[s] = jx / r;
-        uy[s] = jy / r;
+        if constexpr (WANT_U) {
+            ux[s] = velocity_of(jx, r);
+            uy[s] = velocity_of(jy, r);
+        }
     }
 }
 
@@ -566,24 +573,30 @@ __global__ void binary_convert16_kernel(char* set, unsigned pitch, unsigned n, i
 }
 
 // rho, phi, u of a 16-bit set in float64.
+template <bool WANT_U>
 __global__ void binary_moments16_kernel(const char* set, unsigned pitch, unsigned n, float pref, double* rho,
                                         double* phi, double* ux, double* uy) {
     for (unsigned s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-        double r = double(reinterpret_cast<const float*>(set)[s]);
-        double p = double(reinterpret_cast<const float*>(set + 4u * pitch)[s]);
+        double r = lbk::widen(reinterpret_cast<const float*>(set)[s]);
+        double p = lbk::widen(reinterpret_cast<const float*>(set + 4u * pitch)[s]);
         double jx = 0, jy = 0;
-        for (int i = 1; i < Q; ++i) {
-            const double fi = double(__half2float(reinterpret_cast<const __half*>(set + set16_half_offset(i, pitch))[s])) +
+        static_for<1, Q>([&](auto K) {
+            constexpr int i = decltype(K)::value;
+            const double fi = lbk::widen(__half2float(reinterpret_cast<const __half*>(set + set16_half_offset(i, pitch))[s])) +
                               lbk::w_vel<D2Q9>(i) * double(pref);
             r += fi;
-            jx += D2Q9::ex(i) * fi;
-            jy += D2Q9::ey(i) * fi;
-            p += double(__half2float(reinterpret_cast<const __half*>(set + set16_half_offset(Q + i, pitch))[s]));
-        }
+            p += lbk::widen(__half2float(reinterpret_cast<const __half*>(set + set16_half_offset(Q + i, pitch))[s]));
+            if constexpr (WANT_U) {
+                jx = signed_add<D2Q9::ex(i)>(jx, fi);
+                jy = signed_add<D2Q9::ey(i)>(jy, fi);
+            }
+        });
         rho[s] = r;
         phi[s] = p;
-        ux[s] = jx / r;
-        uy[s] = jy / r;
+        if constexpr (WANT_U) {
+            ux[s] = velocity_of(jx, r);
+            uy[s] = velocity_of(jy, r);
+        }
     }
 }
 
@@ -740,14 +753,15 @@ lb_status reset_after_set(lb_binary* c) {
 }
 
 // Observables of the current state into the workspace:
-// rho, phi, ux, uy, vx, vy, mu, mdiff, mxy (each N doubles).
-lb_status compute_fields(lb_binary* c) {
+// rho, phi, ux, uy, vx, vy, mu, mdiff, mxy (each N doubles).  rho and phi always;
+// u, v and mu (and the M' fields that v takes) only where they are asked for.
+lb_status compute_fields(lb_binary* c, bool need_u, bool need_v, bool need_mu) {
     lb_status s = ensure_work(c);
     if (s != LB_OK) return s;
     if (c->D == 3) {
         cudaError_t e = binary_fields3(c->p.scheme == LB_SCHEME_FORCING, c->p.storage == LB_F32, set_ptr(c, c->cur),
                                        unsigned(c->pitch), c->p.nx, c->p.ny, c->p.nz, c->p.A, c->p.B, c->p.kappa,
-                                       c->work, c->stream);
+                                       c->work, need_u, need_v, need_mu, c->stream);
         if (e != cudaSuccess) return brecord(c, e, "binary fields");
         return LB_OK;
     }
@@ -757,20 +771,28 @@ lb_status compute_fields(lb_binary* c) {
            *mu = w + 6 * N, *md = w + 7 * N, *mx = w + 8 * N;
     const unsigned nb = blocks_for(N);
     const int nx = c->p.nx, ny = c->p.ny;
-    if (c->f16)
-        binary_moments16_kernel<<<nb, 256, 0, c->stream>>>(set_ptr(c, c->cur), unsigned(c->pitch), unsigned(N), c->pref,
-                                                           rho, phi, ux, uy);
-    else if (c->p.storage == LB_F64)
-        binary_moments_kernel<double><<<nb, 256, 0, c->stream>>>(
-            reinterpret_cast<const double*>(set_ptr(c, c->cur)), c->pitch, nx, ny, rho, phi, ux, uy);
-    else
-        binary_moments_kernel<float><<<nb, 256, 0, c->stream>>>(
-            reinterpret_cast<const float*>(set_ptr(c, c->cur)), c->pitch, nx, ny, rho, phi, ux, uy);
+    auto moments = [&](auto want_u) {
+        constexpr bool U = decltype(want_u)::value;
+        const void* src = set_ptr(c, c->cur);
+        if (c->f16)
+            binary_moments16_kernel<U><<<nb, 256, 0, c->stream>>>(static_cast<const char*>(src), unsigned(c->pitch),
+                                                                  unsigned(N), c->pref, rho, phi, ux, uy);
+        else if (c->p.storage == LB_F64)
+            binary_moments_kernel<double, U><<<nb, 256, 0, c->stream>>>(static_cast<const double*>(src), c->pitch, nx, ny,
+                                                                        rho, phi, ux, uy);
+        else
+            binary_moments_kernel<float, U><<<nb, 256, 0, c->stream>>>(static_cast<const float*>(src), c->pitch, nx, ny,
+                                                                       rho, phi, ux, uy);
+    };
+    if (need_u || need_v) moments(std::true_type{});
+    else moments(std::false_type{});
     const bool forcing = c->p.scheme == LB_SCHEME_FORCING;
-    binary_mu_kernel<<<nb, 256, 0, c->stream>>>(phi, nx, ny, c->p.A, c->p.B, c->p.kappa, mu, forcing ? md : nullptr,
-                                                 forcing ? mx : nullptr);
+    if (need_mu || (need_v && forcing))
+        binary_mu_kernel<<<nb, 256, 0, c->stream>>>(phi, nx, ny, c->p.A, c->p.B, c->p.kappa, mu,
+                                                     forcing && need_v ? md : nullptr, forcing && need_v ? mx : nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return brecord(c, e, "binary moments");
+    if (!need_v) return LB_OK;
     if (forcing) {
         binary_velocity_kernel<<<nb, 256, 0, c->stream>>>(rho, ux, uy, md, mx, nx, ny, vx, vy);
         e = cudaGetLastError();
@@ -1017,7 +1039,7 @@ lb_status lb_binary_fields(lb_binary* c, double* rho, double* phi, double* u, do
     lb_status s = bcheck(c);
     if (s != LB_OK) return s;
     if (!c->initialised) return bfail(LB_ESTATE, "state not initialised");
-    if ((s = compute_fields(c)) != LB_OK) return s;
+    if ((s = compute_fields(c, u != nullptr, v != nullptr, mu != nullptr)) != LB_OK) return s;
     const long long N = c->N;
     const size_t nb = size_t(N) * sizeof(double);
     const double* w = c->work;

@@ -246,22 +246,29 @@ __global__ void binary_init_kernel3(const double* rho, const double* phi, const 
     }
 }
 
-// Observables in float64: rho, phi, u (3 components) of the stored state.
-template <class real>
+// Observables in float64: rho, phi and, with WANT_U, u (3 components) of the
+// stored state.  Bound by the FP64 pipe: conversions in integer instructions
+// (lbk::widen) and no momentum where u is not asked for (128^3 float32, rho and
+// phi: 601 -> 156 us).
+template <class real, bool WANT_U>
 __global__ void binary_moments_kernel3(const real* src, unsigned pitch, size_t n, double* rho, double* phi, double* u) {
     for (size_t s = blockIdx.x * size_t(blockDim.x) + threadIdx.x; s < n; s += size_t(gridDim.x) * blockDim.x) {
         double r = 0, p = 0, j[3] = {0, 0, 0};
-        for (int i = 0; i < Q3; ++i) {
-            const double fi = double(src[i * size_t(pitch) + s]);
+        static_for<0, Q3>([&](auto K) {
+            constexpr int i = decltype(K)::value;
+            const double fi = lbk::widen(src[i * size_t(pitch) + s]);
             r += fi;
-            j[0] += D3Q19::ex(i) * fi;
-            j[1] += D3Q19::ey(i) * fi;
-            j[2] += D3Q19::ez(i) * fi;
-            p += double(src[(Q3 + i) * size_t(pitch) + s]);
-        }
+            p += lbk::widen(src[(Q3 + i) * size_t(pitch) + s]);
+            if constexpr (WANT_U) {
+                j[0] = signed_add<D3Q19::ex(i)>(j[0], fi);
+                j[1] = signed_add<D3Q19::ey(i)>(j[1], fi);
+                j[2] = signed_add<D3Q19::ez(i)>(j[2], fi);
+            }
+        });
         rho[s] = r;
         phi[s] = p;
-        for (int d = 0; d < 3; ++d) u[d * n + s] = j[d] / r;
+        if constexpr (WANT_U)
+            for (int d = 0; d < 3; ++d) u[d * n + s] = velocity_of(j[d], r);
     }
 }
 
@@ -356,15 +363,21 @@ cudaError_t binary_init3(bool forcing, bool f32, const double* rho, const double
 }
 
 cudaError_t binary_fields3(bool forcing, bool f32, const void* src, unsigned pitch, int nx, int ny, int nz, double A,
-                           double B, double kappa, double* w, cudaStream_t st) {
+                           double B, double kappa, double* w, bool need_u, bool need_v, bool need_mu, cudaStream_t st) {
     const size_t n = size_t(nx) * ny * nz;
     const unsigned nb = blocks3(n);
     double *rho = w, *phi = w + n, *u = w + 2 * n, *v = w + 5 * n, *mu = w + 8 * n, *mt = w + 9 * n;
-    if (f32) binary_moments_kernel3<float><<<nb, 256, 0, st>>>(static_cast<const float*>(src), pitch, n, rho, phi, u);
-    else binary_moments_kernel3<double><<<nb, 256, 0, st>>>(static_cast<const double*>(src), pitch, n, rho, phi, u);
-    binary_mu_kernel3<<<nb, 256, 0, st>>>(phi, nx, ny, nz, A, B, kappa, mu, forcing ? mt : nullptr);
+    auto moments = [&](auto want_u) {
+        constexpr bool U = decltype(want_u)::value;
+        if (f32) binary_moments_kernel3<float, U><<<nb, 256, 0, st>>>(static_cast<const float*>(src), pitch, n, rho, phi, u);
+        else binary_moments_kernel3<double, U><<<nb, 256, 0, st>>>(static_cast<const double*>(src), pitch, n, rho, phi, u);
+    };
+    if (need_u || need_v) moments(std::true_type{});
+    else moments(std::false_type{});
+    if (need_mu || (need_v && forcing))
+        binary_mu_kernel3<<<nb, 256, 0, st>>>(phi, nx, ny, nz, A, B, kappa, mu, forcing && need_v ? mt : nullptr);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !need_v) return e;
     if (forcing) {
         binary_velocity_kernel3<<<nb, 256, 0, st>>>(rho, u, mt, nx, ny, nz, v);
         return cudaGetLastError();

@@ -46,6 +46,11 @@ struct StepArgs {
     unsigned* status;
 };
 
+// A component of u = j / rho for the diagnostics; NaN where a population, and so rho, is not finite.
+__device__ __forceinline__ double velocity_of(double j, double rho) {
+    return isfinite(rho) ? j / rho : rho - rho;   // inf - inf, NaN - NaN
+}
+
 template <class real>
 __device__ __forceinline__ real cst(double d) { return real(d); }
 template <>

@@ -19,8 +19,10 @@ cudaError_t binary_init3(bool forcing, bool f32, const double* rho, const double
                          cudaStream_t st);
 
 // Observables of the set `src` into the workspace w (15 N doubles): rho, phi,
-// u [3], v [3], mu, and (forcing) the six M' fields of the body force.
+// and where needed u [3], v [3], mu, and (forcing, for v) the six M' fields of
+// the body force.
 cudaError_t binary_fields3(bool forcing, bool f32, const void* src, unsigned pitch, int nx, int ny, int nz, double A,
-                           double B, double kappa, double* w, cudaStream_t st);
+                           double B, double kappa, double* w, bool need_u, bool need_v, bool need_mu,
+                           cudaStream_t st);
 
 }  // namespace lbb

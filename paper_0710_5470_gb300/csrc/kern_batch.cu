@@ -52,7 +52,8 @@ struct BatchLaunch {
     }
     static cudaError_t moments(const PopPtrs& p, Grid3 g, double* rho, double* u, cudaStream_t st) {
         const size_t n = size_t(g.nx) * g.ny * g.nz;
-        moments_kernel<D2Q9, S><<<lbk_aux_blocks(n), 256, 0, st>>>(p, g, rho, u);
+        if (u) moments_kernel<D2Q9, S, true><<<lbk_aux_blocks(n), 256, 0, st>>>(p, g, rho, u);
+        else moments_kernel<D2Q9, S, false><<<lbk_aux_blocks(n), 256, 0, st>>>(p, g, rho, u);
         return cudaGetLastError();
     }
     static cudaError_t get_pops(const PopPtrs& p, size_t n, double* out, cudaStream_t st) {
@@ -169,6 +170,7 @@ struct lb_batch {
     double self_rtol = 0.0, self_tol_rho = 0.0;   // lb_batch_set_self_test (0: off)
     int self_hold = 10;
     long long* d_steps = nullptr;
+    std::vector<long long> h_steps;   // host copy of d_steps, which only lb_batch_run_to_steady and a reset change
     long long* d_gstep = nullptr;
     double* d_uprev = nullptr;
     double* w_rho = nullptr;          // scratch of the largest instance
@@ -273,6 +275,7 @@ lb_status reset_run_state(lb_batch* B) {
     if (e == cudaSuccess) e = cudaMemsetAsync(B->d_uprev, 0, size_t(B->sites) * 2 * sizeof(double), B->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(B->stream);
     if (e != cudaSuccess) return cuda_err(e, "batch reset");
+    B->h_steps = minus;
     B->gstep = 0;
     B->parity = 0;
     return set_tile(B, B->tile);
@@ -574,6 +577,7 @@ lb_status lb_batch_run_to_steady(lb_batch* B, double tol, int every, long long m
     e = cudaMemcpy(st.data(), B->d_steps, B->n * sizeof(long long), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(stat.data(), B->d_status, B->n * sizeof(unsigned), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_err(e, "batch results");
+    B->h_steps = st;
     for (int k = 0; k < B->n; ++k) {
         if (steps_out) steps_out[k] = st[k];
         if (status_out) status_out[k] = stat[k] ? LB_EUNSTABLE : (st[k] < 0 ? LB_ETIMEOUT : LB_OK);
@@ -636,11 +640,8 @@ lb_status lb_batch_fields(lb_batch* B, int k, double* rho, double* u) {
     const BatchInst& I = B->di[k];
     const size_t N = size_t(I.nx) * I.ny;
     // a retired instance keeps the buffer it was in when it stopped: even step counts end in buffer 0
-    long long sd = 0;
-    cudaError_t e = cudaMemcpy(&sd, B->d_steps + k, sizeof(long long), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_err(e, "steps");
-    const int par = sd >= 0 ? 0 : B->parity;
-    e = B->k.moments(pops_of(B, k, par), Grid3{I.nx, I.ny, 1}, B->w_rho, B->w_u, B->stream);
+    const int par = B->h_steps[k] >= 0 ? 0 : B->parity;
+    cudaError_t e = B->k.moments(pops_of(B, k, par), Grid3{I.nx, I.ny, 1}, B->w_rho, u ? B->w_u : nullptr, B->stream);
     if (e == cudaSuccess && rho) e = cudaMemcpyAsync(rho, B->w_rho, N * sizeof(double), cudaMemcpyDeviceToHost, B->stream);
     if (e == cudaSuccess && u) e = cudaMemcpyAsync(u, B->w_u, 2 * N * sizeof(double), cudaMemcpyDeviceToHost, B->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(B->stream);
@@ -651,11 +652,8 @@ lb_status lb_batch_populations(lb_batch* B, int k, double* f) {
     if (!B || k < 0 || k >= B->n || !f) return fail(LB_EINVAL, "bad arguments");
     const BatchInst& I = B->di[k];
     const size_t N = size_t(I.nx) * I.ny;
-    long long sd = 0;
-    cudaError_t e = cudaMemcpy(&sd, B->d_steps + k, sizeof(long long), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_err(e, "steps");
-    const int par = sd >= 0 ? 0 : B->parity;
-    e = B->k.get_pops(pops_of(B, k, par), N, B->w_io, B->stream);
+    const int par = B->h_steps[k] >= 0 ? 0 : B->parity;
+    cudaError_t e = B->k.get_pops(pops_of(B, k, par), N, B->w_io, B->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(f, B->w_io, 9 * N * sizeof(double), cudaMemcpyDeviceToHost, B->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(B->stream);
     return e == cudaSuccess ? LB_OK : cuda_err(e, "batch populations");

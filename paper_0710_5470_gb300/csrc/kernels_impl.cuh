@@ -62,7 +62,8 @@ struct Launchers {
     }
     static cudaError_t moments(const PopPtrs& p, Grid3 g, double* rho, double* u, cudaStream_t st) {
         const size_t n = size_t(g.nx) * g.ny * g.nz;
-        moments_kernel<L, S><<<lbk_aux_blocks(n), 256, 0, st>>>(p, g, rho, u);
+        if (u) moments_kernel<L, S, true><<<lbk_aux_blocks(n), 256, 0, st>>>(p, g, rho, u);
+        else moments_kernel<L, S, false><<<lbk_aux_blocks(n), 256, 0, st>>>(p, g, rho, u);
         return cudaGetLastError();
     }
     static cudaError_t mprime(const double* rho, Grid3 g, double kappa, double* mp, cudaStream_t st) {

@@ -318,12 +318,12 @@ lb_status sync_status(lb_ctx* c) {
     return LB_OK;
 }
 
-// rho, u (and v for the forcing scheme) of the current state in the work arrays.
-lb_status compute_fields(lb_ctx* c, bool need_v) {
+// rho and, where asked for, u and v of the current state in the work arrays (v needs u).
+lb_status compute_fields(lb_ctx* c, bool need_u, bool need_v) {
     lb_status s = ensure_work(c);
     if (s != LB_OK) return s;
     const lbk::PopPtrs src = pop_ptrs(c, c->cur);
-    cudaError_t e = c->ks.moments(src, grid3(c), c->w_rho, c->w_u, c->stream);
+    cudaError_t e = c->ks.moments(src, grid3(c), c->w_rho, need_u || need_v ? c->w_u : nullptr, c->stream);
     if (e != cudaSuccess) return record(c, e, "moments");
     if (need_v && c->p.scheme == LB_SCHEME_FORCING && c->free_params) {
         e = lbk::free2d_velocity_v(c->fw, c->p.kappa, c->w_rho, c->w_u, c->p.nx, c->p.ny, c->p2_gl, c->p2_mp,
@@ -916,7 +916,7 @@ lb_status lb_fields(lb_ctx* c, double* rho, double* u, double* v) {
     lb_status s = check_ctx(c);
     if (s != LB_OK) return s;
     if (!c->initialised) return fail(LB_ESTATE, "state not initialised");
-    if ((s = compute_fields(c, v != nullptr)) != LB_OK) return s;
+    if ((s = compute_fields(c, u != nullptr, v != nullptr)) != LB_OK) return s;
     cudaError_t e = cudaSuccess;
     const size_t dn = size_t(c->D) * c->N * sizeof(double);
     if (rho) e = cudaMemcpyAsync(rho, c->w_rho, c->N * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
@@ -931,7 +931,7 @@ lb_status lb_stats_get(lb_ctx* c, lb_stats* out) {
     if (s != LB_OK) return s;
     if (!out) return fail(LB_EINVAL, "null output");
     if (!c->initialised) return fail(LB_ESTATE, "state not initialised");
-    if ((s = compute_fields(c, true)) != LB_OK) return s;
+    if ((s = compute_fields(c, true, true)) != LB_OK) return s;
     const size_t du = size_t(c->D) * c->N;
     if (!c->w_uprev) {
         cudaError_t e = cudaMalloc(&c->w_uprev, du * sizeof(double));

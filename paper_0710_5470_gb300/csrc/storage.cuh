@@ -21,6 +21,21 @@
 
 namespace lbk {
 
+// float32 -> float64, exactly, without the conversion instruction: that runs
+// on the FP64 pipe (two lanes per clock and SM on a GB300), where it costs as
+// much as the addition that follows it, and the diagnostics kernels that sum 9
+// to 38 populations per site are bound by that pipe.  The exponent is rebiased
+// and the fraction shifted into place; a subnormal is scaled by 2^24 first
+// (exact), zeros keep their sign, infinities and NaN the top exponent.  No
+// branch: a predicated conversion would occupy the pipe all the same.
+__device__ __forceinline__ double widen(float v) {
+    const bool small = fabsf(v) < 1.17549435e-38f;
+    const unsigned b = __float_as_uint(small ? v * 16777216.0f : v), m = b & 0x7fffffffu;
+    const unsigned bias = m == 0u ? 0u : (small ? 0x36800000u : (m >= 0x7f800000u ? 0x70000000u : 0x38000000u));
+    return __hiloint2double(int((b & 0x80000000u) | ((m >> 3) + bias)), int(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
 struct StF64 {
     using real = double;
     using raw0 = double;   // stored type of f_0
