@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "storage.cuh"   // lbk::widen
+
 namespace {
 
 __device__ __forceinline__ int wrap(int v, int n) {
@@ -13,35 +15,43 @@ __device__ __forceinline__ int wrap(int v, int n) {
     return v < 0 ? v + n : v;
 }
 
-// dy = 2 (y - t) / count; loss += sum (y - t)^2 / count (float64 accumulation).
+// dy = 2 (y - t) / count; loss += sum (y - t)^2 / count (float64 accumulation;
+// launched with 256 threads).
 __global__ void mse_grad(const float* y, const float* t, float* dy, size_t n, double* loss) {
-    __shared__ double red[256];
+    __shared__ double red[8];
     double acc = 0.0;
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
         const float d = y[i] - t[i];
         dy[i] = 2.f * d / float(n);
-        acc += double(d) * double(d);
+        const double e = lbk::widen(d);
+        acc += e * e;
     }
-    red[threadIdx.x] = acc;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, s);
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = acc;
     __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (int(threadIdx.x) < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double sum = red[0];
+        for (int k = 1; k < 8; ++k) sum += red[k];
+        atomicAdd(loss, sum / double(n));
     }
-    if (threadIdx.x == 0) atomicAdd(loss, red[0] / double(n));
+}
+
+// One Adam step of parameter i; returns its new value.
+__device__ __forceinline__ float adam_one(float* w, const float* g, float* m, float* v, int i, float lr, float b1,
+                                          float b2, float eps, float c1, float c2) {
+    const float gi = g[i];
+    const float mi = b1 * m[i] + (1.f - b1) * gi;
+    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    return w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
 __global__ void adam_update(float* w, __half* w16, const float* g, float* m, float* v, int n, float lr, float b1,
                             float b2, float eps, float c1, float c2) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-        w16[i] = __float2half_rn(w[i]);
-    }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        w16[i] = __float2half_rn(adam_one(w, g, m, v, i, lr, b1, b2, eps, c1, c2));
 }
 
 __global__ void to_half(const float* w, __half* w16, int n) {
