@@ -8,6 +8,7 @@
 // work list on the device.  No kernel waits on another CTA.
 #pragma once
 #include "aux_kernels.cuh"
+#include "step2d_f64.cuh"
 #include "step2d_pk.cuh"
 
 namespace lbk {
@@ -21,6 +22,7 @@ struct BatchInst {
     double a, b, T, kappa, omega, nu;
     float fa, fb, fT, fkappa, fomega, fnu;   // their float32 roundings
     float pref, rsum;
+    Consts64 c64;          // float64 storage
 };
 
 struct BatchState {
@@ -59,8 +61,12 @@ __global__ void __launch_bounds__(TX* TY) batch_step_kernel(BatchState bs, char*
                      I.kappa, I.omega, I.nu, I.fa, I.fb, I.fT, I.fkappa, I.fomega, I.fnu, I.pref, I.rsum,
                      bs.status + k};
         const int tx = I.tiles_x;
-        step2d_tile<D2Q9, FORCING, S, TX, TY>(a, (t % tx) * TX, (t / tx) * TY,
-                                              reinterpret_cast<typename S::real*>(smem_raw));
+        if constexpr (sizeof(typename S::real) == 8)
+            step2d_tile_f64<FORCING, TX, TY, TX * TY>(a, I.c64, (t % tx) * TX, (t / tx) * TY,
+                                                      reinterpret_cast<double*>(smem_raw));
+        else
+            step2d_tile<D2Q9, FORCING, S, TX, TY>(a, (t % tx) * TX, (t / tx) * TY,
+                                                  reinterpret_cast<typename S::real*>(smem_raw));
         __syncthreads();   // shared memory is reused by the next item
     }
 }

@@ -34,7 +34,7 @@ struct LbKernelSet {
 };
 
 // scheme: 0 equilibrium, 1 forcing; storage: lb_storage value.
-LbKernelSet lbk_kernels_d2q9(int scheme, int storage);
+LbKernelSet lbk_kernels_d2q9(int scheme, int storage, int nx, int ny, int sms);
 LbKernelSet lbk_kernels_d3q19(int scheme, int storage, int nx);
 
 // Grid size of the grid-stride auxiliary kernels.

@@ -37,9 +37,10 @@ struct BatchKernels {
 
 template <bool F, class S, int TX, int TY>
 struct BatchLaunch {
-    using Lay = StepLayout<D2Q9, F, TX, TY, typename S::real>;
+    static constexpr size_t BYTES = sizeof(typename S::real) == 8 ? Layout64<F, TX, TY, TX * TY>::BYTES
+                                                                   : StepLayout<D2Q9, F, TX, TY, typename S::real>::BYTES;
     static void step(const BatchState& bs, char* buf, int parity, int nblocks, cudaStream_t st) {
-        batch_step_kernel<F, S, TX, TY><<<nblocks, TX * TY, Lay::BYTES, st>>>(bs, buf, parity);
+        batch_step_kernel<F, S, TX, TY><<<nblocks, TX * TY, BYTES, st>>>(bs, buf, parity);
     }
     static void check(const BatchState& bs, const char* buf, int parity, int nblocks, cudaStream_t st) {
         batch_check_kernel<S, TX, TY><<<nblocks, TX * TY, 0, st>>>(bs, buf, parity);
@@ -65,7 +66,7 @@ struct BatchLaunch {
         k.tx = TX;
         k.ty = TY;
         k.threads = k.check_threads = TX * TY;
-        k.smem = Lay::BYTES;
+        k.smem = BYTES;
         k.step_fn = reinterpret_cast<const void*>(batch_step_kernel<F, S, TX, TY>);
         k.check_fn = reinterpret_cast<const void*>(batch_check_kernel<S, TX, TY>);
         k.step = &step;
@@ -351,6 +352,7 @@ lb_status lb_batch_create(int scheme, int storage, double a, double b, int n, co
         I.fkappa = float(I.kappa);
         I.fomega = float(I.omega);
         I.fnu = float(I.nu);
+        I.c64 = consts64(a, b, in.T, in.kappa, I.omega, I.nu);
         const double rl = B->rho_l[k];
         const double pref = (storage == LB_F16DEV || storage == LB_BF16DEV) ? rl * in.T / (1 - b * rl) - a * rl * rl : 0.0;
         // sum_{i>=1} w_i (5/3 on D2Q9), summed in velocity order like a single

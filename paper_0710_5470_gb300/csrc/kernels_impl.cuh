@@ -2,32 +2,41 @@
 // combination; included by one translation unit per lattice.
 #pragma once
 #include "dispatch.h"
+#include "step2d_f64.cuh"
 #include "step3d.cuh"
 
 namespace lbk {
 
+inline Tile2DArgs tile2d_args(const StepArgs& a) {
+    return Tile2DArgs{a.src_base, a.dst_base, a.pitch, a.nx, a.ny, a.pair2d, a.a, a.b, a.T, a.kappa, a.omega,
+                      a.nu, a.fa, a.fb, a.fT, a.fkappa, a.fomega, a.fnu, a.pref, a.rsum, a.status};
+}
+
 // Fused step kernel of a lattice: the z-split kernel for D3Q19 (PAIR: two
-// sites per stage-A load, even nx only), the generic single-plane kernel for
-// D2Q9 (PAIR ignored).
+// sites per stage-A load, even nx only), the single-plane kernel for D2Q9
+// (PAIR ignored; float64 arithmetic: step2d_f64.cuh).
 template <class L, bool FORCING, class S, int TX, int TY, bool PAIR = false>
 struct StepKernelOf {
     using real = typename S::real;
-    static constexpr bool D3 = L::D == 3;
+    static constexpr bool D3 = L::D == 3, F64 = sizeof(real) == 8;
     static constexpr size_t bytes() {
-        if constexpr (D3) return Layout3D<FORCING, TX, TY, real, sizeof(typename S::rawi) == 2>::BYTES;
+        if constexpr (!D3 && F64) return Layout64<FORCING, TX, TY, TX * TY>::BYTES;
+        else if constexpr (D3) return Layout3D<FORCING, TX, TY, real, sizeof(typename S::rawi) == 2>::BYTES;
         else return StepLayout<L, FORCING, TX, TY, real>::BYTES;
     }
     static const void* fn() {
-        if constexpr (D3) return reinterpret_cast<const void*>(step_kernel3d<FORCING, S, TX, TY, PAIR>);
+        if constexpr (!D3 && F64) return reinterpret_cast<const void*>(step_kernel2d_f64<FORCING, TX, TY, TX * TY>);
+        else if constexpr (D3) return reinterpret_cast<const void*>(step_kernel3d<FORCING, S, TX, TY, PAIR>);
         else return reinterpret_cast<const void*>(step_kernel<L, FORCING, S, TX, TY>);
     }
     static void launch(dim3 grid, cudaStream_t st, const StepArgs& a) {
         if constexpr (D3) {
             step_kernel3d<FORCING, S, TX, TY, PAIR><<<grid, TX * TY, bytes(), st>>>(a);
+        } else if constexpr (F64) {
+            step_kernel2d_f64<FORCING, TX, TY, TX * TY><<<grid, TX * TY, bytes(), st>>>(
+                tile2d_args(a), consts64(a.a, a.b, a.T, a.kappa, a.omega, a.nu));
         } else {
-            Tile2DArgs t{a.src_base, a.dst_base, a.pitch, a.nx, a.ny, a.pair2d, a.a, a.b, a.T, a.kappa, a.omega,
-                         a.nu, a.fa, a.fb, a.fT, a.fkappa, a.fomega, a.fnu, a.pref, a.rsum, a.status};
-            step_kernel<L, FORCING, S, TX, TY><<<grid, TX * TY, bytes(), st>>>(t);
+            step_kernel<L, FORCING, S, TX, TY><<<grid, TX * TY, bytes(), st>>>(tile2d_args(a));
         }
     }
 };

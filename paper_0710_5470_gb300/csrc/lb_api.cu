@@ -539,7 +539,10 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
     const int elem0 = p->storage == LB_F64 ? 8 : 4;
     const int elemi = p->storage == LB_F64 ? 8 : (p->storage == LB_F32 ? 4 : 2);
     c->buf_bytes = c->pitch * (elem0 + size_t(c->Q - 1) * elemi);
-    c->ks = c->D == 2 ? lbk_kernels_d2q9(p->scheme, p->storage) : lbk_kernels_d3q19(p->scheme, p->storage, p->nx);
+    int dev = 0, sms = 0, occ = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    c->ks = c->D == 2 ? lbk_kernels_d2q9(p->scheme, p->storage, p->nx, p->ny, sms) : lbk_kernels_d3q19(p->scheme, p->storage, p->nx);
     if (!c->ks.step) { delete c; return fail(LB_EINVAL, "no kernel for this combination"); }
     // two sites per halo load need an even nx; LB_NO_PAIR selects the
     // one-site form (same arithmetic) everywhere, for comparison
@@ -574,9 +577,6 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
 
     // launch geometry of the fused step: one CTA per TX x TY column tile and z chunk;
     // the z chunk is sized so that all CTAs are resident at once where possible.
-    int dev = 0, sms = 0, occ = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncSetAttribute(c->ks.step_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(c->ks.smem));
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, c->ks.step_fn, c->ks.threads, c->ks.smem) !=
             cudaSuccess || occ < 1)
