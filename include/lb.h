@@ -111,6 +111,8 @@ lb_status lb_coexistence(double a, double b, double T, double* rho_l, double* rh
  * allocates the two population buffers on the current CUDA device.
  * cuda_stream is a cudaStream_t (NULL = the legacy default stream); it must
  * outlive the context.  *out receives the context, or NULL on error.
+ * D3Q19 float64 contexts also allocate a workspace of 11 (forcing scheme) or 1
+ * float64 per site, at most 1 GiB; where it cannot be had they step without it.
  * LB_EINVAL also for more than 2^31 - 1 sites (the kernels index sites with
  * 32-bit integers). */
 lb_status lb_create(const lb_params* p, void* cuda_stream, lb_ctx** out);

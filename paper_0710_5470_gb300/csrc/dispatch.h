@@ -37,6 +37,12 @@ struct LbKernelSet {
 LbKernelSet lbk_kernels_d2q9(int scheme, int storage, int nx, int ny, int sms);
 LbKernelSet lbk_kernels_d3q19(int scheme, int storage, int nx);
 
+// The float64 D3Q19 step in passes (kern_d3q19_f64.cu): planes per slab and bytes
+// of its workspace (0: no slab of a useful depth fits the workspace's limit; the
+// fused kernel steps such a lattice), and `k` with its step.
+int lbk_f64_slab(int scheme, int nx, int ny, int nz, size_t* bytes);
+LbKernelSet lbk_f64_passes(int scheme, LbKernelSet k);
+
 // Grid size of the grid-stride auxiliary kernels.
 inline unsigned lbk_aux_blocks(size_t n) {
     size_t b = (n + 255) / 256;

@@ -119,6 +119,7 @@ struct lb_ctx {
     int lz = 1;
     dim3 grid;
     int4* d_work = nullptr;   // 3D: per-CTA (x0, y0, z0, z1)
+    double* work64 = nullptr; // float64 D3Q19 in passes: workspace of `lz` planes per slab
     bool initialised = false;
     long long step = 0;
     lb_status sticky = LB_OK;
@@ -444,6 +445,7 @@ unsigned long long lbk_bounds_d2q9();
 unsigned long long lbk_bounds_d2pk();
 unsigned long long lbk_bounds_d3pke();
 unsigned long long lbk_bounds_batch();
+unsigned long long lbk_bounds_d3f64();
 
 extern "C" {
 
@@ -582,19 +584,34 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
             cudaSuccess || occ < 1)
         occ = 1;
     cudaGetLastError();
-    const int gx = (p->nx + c->ks.tx - 1) / c->ks.tx;
-    const int gy = (p->ny + c->ks.ty - 1) / c->ks.ty;
-    c->lz = 1;
-    c->grid = dim3(gx, gy, 1);
-    if (c->D == 3) {
-        const std::vector<int4> work = build_work_list(sms, occ, p->nx, p->ny, p->nz, c->ks.tx, c->ks.ty);
-        c->lz = work.front().w - work.front().z;
-        if (cudaMalloc(&c->d_work, work.size() * sizeof(int4)) != cudaSuccess ||
-            cudaMemcpy(c->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess) {
-            lb_destroy(c);
-            return fail(LB_ENOMEM, "work list");
+    // float64 D3Q19: in passes where their workspace is to be had, else the fused kernel
+    if (c->D == 3 && p->storage == LB_F64) {
+        size_t bytes = 0;
+        const int slab = lbk_f64_slab(p->scheme, p->nx, p->ny, p->nz, &bytes);
+        if (slab > 0 && cudaMalloc(&c->work64, bytes) == cudaSuccess) {
+            c->ks = lbk_f64_passes(p->scheme, c->ks);
+            c->lz = slab;
+            c->grid = dim3(unsigned((size_t(p->nx) * p->ny * std::min(slab, p->nz) + c->ks.threads - 1) / c->ks.threads));
+        } else {
+            c->work64 = nullptr;
+            cudaGetLastError();
         }
-        c->grid = dim3(unsigned(work.size()), 1, 1);
+    }
+    if (!c->work64) {
+        const int gx = (p->nx + c->ks.tx - 1) / c->ks.tx;
+        const int gy = (p->ny + c->ks.ty - 1) / c->ks.ty;
+        c->lz = 1;
+        c->grid = dim3(gx, gy, 1);
+        if (c->D == 3) {
+            const std::vector<int4> work = build_work_list(sms, occ, p->nx, p->ny, p->nz, c->ks.tx, c->ks.ty);
+            c->lz = work.front().w - work.front().z;
+            if (cudaMalloc(&c->d_work, work.size() * sizeof(int4)) != cudaSuccess ||
+                cudaMemcpy(c->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess) {
+                lb_destroy(c);
+                return fail(LB_ENOMEM, "work list");
+            }
+            c->grid = dim3(unsigned(work.size()), 1, 1);
+        }
     }
     c->probe_in[0] = p->nx / 2;
     c->probe_in[1] = p->ny / 2;
@@ -620,6 +637,7 @@ lb_status lb_destroy(lb_ctx* c) {
     cudaFree(c->w_io);
     cudaFree(c->w_uprev);
     cudaFree(c->d_work);
+    cudaFree(c->work64);
     cudaFree(c->p2_rho);
     cudaFree(c->p2_gl);
     cudaFree(c->p2_mp);
@@ -835,6 +853,7 @@ lb_status lb_step(lb_ctx* c, int nsteps) {
     a.nz = c->p.nz;
     a.lz = c->lz;
     a.work = c->d_work;
+    a.work64 = c->work64;
     a.pair2d = (c->D == 2 && c->p.nx % 2 == 0 && !std::getenv("LB_NO_PAIR")) ? 1 : 0;
     a.a = c->p.a;
     a.b = c->p.b;
@@ -1004,7 +1023,7 @@ lb_status lb_debug_bounds(int* checked, unsigned long long* violation) {
     if (checked) *checked = lbk::kBoundsChecked ? 1 : 0;
     unsigned long long v = 0;
     for (unsigned long long w : {lbk_bounds_d3pk(), lbk_bounds_d3pke(), lbk_bounds_d3q19(), lbk_bounds_d2q9(), lbk_bounds_d2pk(),
-                                 lbk_bounds_batch()})
+                                 lbk_bounds_batch(), lbk_bounds_d3f64()})
         if (!v) v = w;
     if (violation) *violation = v;
     return LB_OK;
