@@ -43,6 +43,12 @@ LbKernelSet lbk_kernels_d3q19(int scheme, int storage, int nx);
 int lbk_f64_slab(int scheme, int nx, int ny, int nz, size_t* bytes);
 LbKernelSet lbk_f64_passes(int scheme, LbKernelSet k);
 
+// The two-pass forcing step of 32-bit arithmetic (kern_d3q19_fd.cu) in place of
+// the step of `k`, for the lattices that lbk_fd_wanted names; it needs a density
+// field of one float32 per site.
+bool lbk_fd_wanted(int storage, int nx, size_t sites);
+LbKernelSet lbk_fd_forcing(int storage, int nx, LbKernelSet k);
+
 // Grid size of the grid-stride auxiliary kernels.
 inline unsigned lbk_aux_blocks(size_t n) {
     size_t b = (n + 255) / 256;

@@ -119,6 +119,7 @@ struct lb_ctx {
     int lz = 1;
     dim3 grid;
     int4* d_work = nullptr;   // 3D: per-CTA (x0, y0, z0, z1)
+    float* rho32 = nullptr;   // D3Q19 in two passes: density field (pitch float32)
     double* work64 = nullptr; // float64 D3Q19 in passes: workspace of `lz` planes per slab
     bool initialised = false;
     long long step = 0;
@@ -446,6 +447,7 @@ unsigned long long lbk_bounds_d2pk();
 unsigned long long lbk_bounds_d3pke();
 unsigned long long lbk_bounds_batch();
 unsigned long long lbk_bounds_d3f64();
+unsigned long long lbk_bounds_d3fd();
 
 extern "C" {
 
@@ -577,6 +579,17 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
     }
     cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream);
 
+    // D3Q19 forcing scheme in 32 bits: in two passes where that is faster and a density
+    // field is to be had, else the fused kernel (the layout of the populations is the same)
+    if (c->D == 3 && p->scheme == LB_SCHEME_FORCING && p->storage != LB_F64 && !std::getenv("LB_D3_VARIANT") &&
+        !std::getenv("LB_NO_PAIR") && lbk_fd_wanted(p->storage, p->nx, c->N)) {
+        if (cudaMalloc(&c->rho32, c->pitch * sizeof(float)) == cudaSuccess) {
+            c->ks = lbk_fd_forcing(p->storage, p->nx, c->ks);
+        } else {
+            c->rho32 = nullptr;
+            cudaGetLastError();
+        }
+    }
     // launch geometry of the fused step: one CTA per TX x TY column tile and z chunk;
     // the z chunk is sized so that all CTAs are resident at once where possible.
     cudaFuncSetAttribute(c->ks.step_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(c->ks.smem));
@@ -638,6 +651,7 @@ lb_status lb_destroy(lb_ctx* c) {
     cudaFree(c->w_uprev);
     cudaFree(c->d_work);
     cudaFree(c->work64);
+    cudaFree(c->rho32);
     cudaFree(c->p2_rho);
     cudaFree(c->p2_gl);
     cudaFree(c->p2_mp);
@@ -854,6 +868,7 @@ lb_status lb_step(lb_ctx* c, int nsteps) {
     a.lz = c->lz;
     a.work = c->d_work;
     a.work64 = c->work64;
+    a.rho32 = c->rho32;
     a.pair2d = (c->D == 2 && c->p.nx % 2 == 0 && !std::getenv("LB_NO_PAIR")) ? 1 : 0;
     a.a = c->p.a;
     a.b = c->p.b;
@@ -1023,7 +1038,7 @@ lb_status lb_debug_bounds(int* checked, unsigned long long* violation) {
     if (checked) *checked = lbk::kBoundsChecked ? 1 : 0;
     unsigned long long v = 0;
     for (unsigned long long w : {lbk_bounds_d3pk(), lbk_bounds_d3pke(), lbk_bounds_d3q19(), lbk_bounds_d2q9(), lbk_bounds_d2pk(),
-                                 lbk_bounds_batch(), lbk_bounds_d3f64()})
+                                 lbk_bounds_batch(), lbk_bounds_d3f64(), lbk_bounds_d3fd()})
         if (!v) v = w;
     if (violation) *violation = v;
     return LB_OK;

@@ -406,6 +406,67 @@ struct LayoutPK {
     __host__ __device__ static constexpr int mp_index(int sx, int sy) { return (sx & 1) * (SY * SXH) + sy * SXH + (sx >> 1); }
 };
 
+// Body force of the own pair (Eq. 28): the parts of plane q of M' added to the
+// carries -(U0(q-1) + U-(q-2)) and -U-(q-1); gf: the force of plane q - 1.  (cx0,
+// cy): ring column left of the pair's site 0, and its ring row.
+template <class Lay>
+__device__ __forceinline__ void pair_force_parts(const float4* mpA, const float2* mpB, int cx0, int cy, P2 (&gacc1)[3],
+                                                 P2 (&gacc2)[3], P2 (&gf)[3]) {
+    // neighbourhood columns c = 0..3 (sites x-1 .. x+2) and rows -1, 0, +1 of the
+    // ring; site 0 of the pair is column 1, site 1 column 2
+    float sp[2][3] = {}, sz[2][3] = {}, se[2][3] = {}, zc[2][3];
+    #pragma unroll
+    for (int r = -1; r <= 1; ++r) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int k = Lay::mp_index(cx0 + c, cy + r);
+            const float4 A = mpA[k];
+            const float2 B = mpB[k];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const int dx = c - 1 - s;   // column offset from site s
+                if (dx < -1 || dx > 1) continue;
+                if (r == 0 && dx == 0) {
+                    zc[s][0] = A.z; zc[s][1] = B.x; zc[s][2] = B.y;
+                } else if (r == 0) {        // x neighbour, sign dx
+                    if (dx > 0) {
+                        sp[s][0] += A.x; sp[s][1] += A.y; sp[s][2] += A.z;
+                    } else {
+                        sp[s][0] -= A.x; sp[s][1] -= A.y; sp[s][2] -= A.z;
+                    }
+                    sz[s][0] += A.z; sz[s][1] += B.x; sz[s][2] += B.y;
+                } else if (dx == 0) {       // y neighbour, sign r
+                    if (r > 0) {
+                        sp[s][0] += A.y; sp[s][1] += A.w; sp[s][2] += B.x;
+                    } else {
+                        sp[s][0] -= A.y; sp[s][1] -= A.w; sp[s][2] -= B.x;
+                    }
+                    sz[s][0] += A.z; sz[s][1] += B.x; sz[s][2] += B.y;
+                } else {                    // xy diagonal (dx, r)
+                    const float ax = dx > 0 ? A.x : -A.x, ay = dx > 0 ? A.y : -A.y, az = dx > 0 ? A.z : -A.z;
+                    const float by = r > 0 ? A.y : -A.y, bw = r > 0 ? A.w : -A.w, bx = r > 0 ? B.x : -B.x;
+                    se[s][0] += ax + by;
+                    se[s][1] += ay + bw;
+                    se[s][2] += az + bx;
+                }
+            }
+        }
+    }
+    constexpr float sixth = 1.0f / 6.0f, twelfth = 1.0f / 12.0f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const P2 SP = pp(sp[0][c], sp[1][c]), SZ = pp(sz[0][c], sz[1][c]), SE = pp(se[0][c], se[1][c]);
+        const P2 ZC = pp(zc[0][c], zc[1][c]);
+        const P2 u0 = fma(pp(sixth), SP, pp(twelfth) * SE);
+        const P2 up = fma(pp(twelfth), SP + SZ, pp(sixth) * ZC);
+        const P2 um = fma(pp(twelfth), SP - SZ, -(pp(sixth) * ZC));
+        // g(q-1) = -(U+(q) + U0(q-1) + U-(q-2))
+        gf[c] = gacc1[c] - up;
+        gacc1[c] = gacc2[c] - u0;
+        gacc2[c] = -um;
+    }
+}
+
 // Byte offset of site q in the interleaved 16-bit layout (PopPtrs aos = 1):
 // blocks of AOS_SITES sites, 18 rows of AOS_SITES values each.
 __host__ __device__ __forceinline__ unsigned aos_bytes(unsigned q) {
@@ -656,60 +717,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk(const St
         // ---------------- body force of the own pair: parts of plane q (Eq. 28)
         P2 gf[3] = {pp(0.f), pp(0.f), pp(0.f)};
         if (assemble) {
-            // neighbourhood columns c = 0..3 (sites x-1 .. x+2) and rows -1, 0, +1 of the
-            // ring; site 0 of the pair is column 1, site 1 column 2
-            float sp[2][3] = {}, sz[2][3] = {}, se[2][3] = {}, zc[2][3];
-            const int cx0 = 2 * px, cy = py + 1;
-#pragma unroll
-            for (int r = -1; r <= 1; ++r) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int k = Lay::mp_index(cx0 + c, cy + r);
-                    const float4 A = mpA[k];
-                    const float2 B = mpB[k];
-#pragma unroll
-                    for (int s = 0; s < 2; ++s) {
-                        const int dx = c - 1 - s;   // column offset from site s
-                        if (dx < -1 || dx > 1) continue;
-                        if (r == 0 && dx == 0) {
-                            zc[s][0] = A.z; zc[s][1] = B.x; zc[s][2] = B.y;
-                        } else if (r == 0) {        // x neighbour, sign dx
-                            if (dx > 0) {
-                                sp[s][0] += A.x; sp[s][1] += A.y; sp[s][2] += A.z;
-                            } else {
-                                sp[s][0] -= A.x; sp[s][1] -= A.y; sp[s][2] -= A.z;
-                            }
-                            sz[s][0] += A.z; sz[s][1] += B.x; sz[s][2] += B.y;
-                        } else if (dx == 0) {       // y neighbour, sign r
-                            if (r > 0) {
-                                sp[s][0] += A.y; sp[s][1] += A.w; sp[s][2] += B.x;
-                            } else {
-                                sp[s][0] -= A.y; sp[s][1] -= A.w; sp[s][2] -= B.x;
-                            }
-                            sz[s][0] += A.z; sz[s][1] += B.x; sz[s][2] += B.y;
-                        } else {                    // xy diagonal (dx, r)
-                            const float ax = dx > 0 ? A.x : -A.x, ay = dx > 0 ? A.y : -A.y, az = dx > 0 ? A.z : -A.z;
-                            const float by = r > 0 ? A.y : -A.y, bw = r > 0 ? A.w : -A.w, bx = r > 0 ? B.x : -B.x;
-                            se[s][0] += ax + by;
-                            se[s][1] += ay + bw;
-                            se[s][2] += az + bx;
-                        }
-                    }
-                }
-            }
-            constexpr float sixth = 1.0f / 6.0f, twelfth = 1.0f / 12.0f;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const P2 SP = pp(sp[0][c], sp[1][c]), SZ = pp(sz[0][c], sz[1][c]), SE = pp(se[0][c], se[1][c]);
-                const P2 ZC = pp(zc[0][c], zc[1][c]);
-                const P2 u0 = fma(pp(sixth), SP, pp(twelfth) * SE);
-                const P2 up = fma(pp(twelfth), SP + SZ, pp(sixth) * ZC);
-                const P2 um = fma(pp(twelfth), SP - SZ, -(pp(sixth) * ZC));
-                // g(q-1) = -(U+(q) + U0(q-1) + U-(q-2))
-                gf[c] = gacc1[c] - up;
-                gacc1[c] = gacc2[c] - u0;
-                gacc2[c] = -um;
-            }
+            pair_force_parts<Lay>(mpA, mpB, 2 * px, py + 1, gacc1, gacc2, gf);
         }
 
         // ---------------- stage C: collide and push plane s = p - 2

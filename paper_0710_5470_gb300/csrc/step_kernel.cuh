@@ -45,6 +45,7 @@ struct StepArgs {
     int nx, ny, nz;
     int lz;  // longest z chunk of a CTA (3D)
     const int4* work;  // 3D: per CTA (x0, y0, z0, z1) of its column tile and z chunk
+    float* rho32;    // D3Q19 in two passes: density field
     double* work64;  // D3Q19 float64 in passes: workspace (lz planes per slab)
     int pair2d;  // 2D: two sites per halo load (nx even, 32-bit arithmetic)
     double a, b, T, kappa, omega, nu;
