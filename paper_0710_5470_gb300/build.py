@@ -22,7 +22,7 @@ LIB_DEBUG = os.path.join(BUILD_DEBUG, "liblb_debug.so")
 SOURCES = ["kern_d2q9.cu", "kern_d2q9_pk.cu", "kern_d3q19.cu", "kern_d3q19_pk.cu", "kern_d3q19_pk_eq.cu", "kern_d3q19_f64.cu",
             "kern_d3q19_fd.cu",
             "kern_batch.cu", "lb_api.cu", "cnn.cu", "cnn3d.cu", "noalloc.cu",
-           "param2d.cu", "peak.cu", "binary2d.cu", "binary3d.cu"]
+           "param2d.cu", "peak.cu", "binary2d.cu", "binary3d.cu", "binary3d_march.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

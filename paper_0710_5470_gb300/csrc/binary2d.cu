@@ -619,6 +619,8 @@ struct lb_binary {
     size_t esize = 8;
     void* pop = nullptr;          // 2 sets x 2 Q populations x pitch elements
     void* phi = nullptr;          // D3Q19: phi of the current set (one value per site, storage type)
+    int4* d_work = nullptr;       // D3Q19 float32, marching step: its CTAs' tiles and z chunks
+    int ctas = 0;
     int cur = 0;                  // set holding the current populations
     bool initialised = false;
     long long step = 0;
@@ -676,7 +678,10 @@ cudaError_t launch_step(lb_binary* c, int from, cudaStream_t st) {
     a.status = c->d_status;
     a.pref = c->pref;
     const bool forcing = c->p.scheme == LB_SCHEME_FORCING;
-    if (c->D == 3) return binary_step3(forcing, a, static_cast<real*>(c->phi), st);
+    if (c->D == 3) {
+        if constexpr (sizeof(real) == 4) return binary_step3(forcing, a, static_cast<float*>(c->phi), st, c->d_work, c->ctas);
+        else return binary_step3(forcing, a, static_cast<double*>(c->phi), st);
+    }
     if constexpr (sizeof(real) == 4) {
         if (c->pair) {   // float32 or 16-bit, even nx: two sites per thread
             const dim3 grid((c->p.nx + PTX_ - 1) / PTX_, (c->p.ny + PTY - 1) / PTY);
@@ -805,6 +810,15 @@ lb_status compute_fields(lb_binary* c, bool need_u, bool need_v, bool need_mu) {
 
 bool is_fin(double v) { return std::isfinite(v); }
 
+// Whether a float32 D3Q19 lattice runs the marching step (LB_B3_MARCH=0 / 1 forces
+// it, for comparisons).  Small lattices give its long CTAs too little to share out:
+// us per step, bricks / march, 32^3 7.2 / 13.3 (forcing) and 5.4 / 10.6 (equilibrium),
+// 48^3 15.7 / 16.3 and 11.3 / 12.7, 64^3 24.4 / 20.9 and 17.4 / 16.4.
+bool march3_wanted(long long sites) {
+    if (const char* e = std::getenv("LB_B3_MARCH")) return std::atoi(e) != 0;
+    return sites >= 150000;
+}
+
 }  // namespace
 
 extern "C" {
@@ -851,6 +865,25 @@ lb_status lb_binary_create(const lb_binary_params* p, void* stream, lb_binary** 
     c->stream = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMalloc(&c->pop, 2 * c->set_bytes);
     if (e == cudaSuccess && c->D == 3) e = cudaMalloc(&c->phi, size_t(c->N) * c->esize);
+    if (e == cudaSuccess && c->D == 3 && p->storage == LB_F32 && march3_wanted(c->N)) {
+        int dev = 0, sms = 1;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int occ = binary_march3_ctas(p->scheme == LB_SCHEME_FORCING, p->nx);
+        lb_work_list(sms, occ, p->nx, p->ny, p->nz, 32, 8, nullptr, 0, &c->ctas);
+        std::vector<int4> work;
+        try {
+            work.resize(size_t(c->ctas));
+        } catch (...) {
+            e = cudaErrorMemoryAllocation;
+        }
+        if (e == cudaSuccess) {
+            lb_work_list(sms, occ, p->nx, p->ny, p->nz, 32, 8, reinterpret_cast<int*>(work.data()), c->ctas, &c->ctas);
+            e = cudaMalloc(&c->d_work, work.size() * sizeof(int4));
+        }
+        if (e == cudaSuccess)
+            e = cudaMemcpy(c->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    }
     if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -870,6 +903,7 @@ lb_status lb_binary_destroy(lb_binary* c) {
     drop_graphs(c);
     cudaFree(c->pop);
     cudaFree(c->phi);
+    cudaFree(c->d_work);
     cudaFree(c->d_status);
     cudaFree(c->work);
     cudaFree(c->d_in);

@@ -4,7 +4,8 @@
 //
 // Two launches per time step:
 //   binary_phi_kernel     phi = sum_i g_i of every site (19 reads, one write);
-//   binary_step_kernel3   one CTA per 32 x 4 x 2 brick, one site per thread:
+//   binary_step_kernel3   (float64, and float32 lattices too small for the marching
+//     step of binary3d_march.cuh) one CTA per 32 x 4 x 2 brick, one site per thread:
 //     the brick's phi plus a halo (1 site for the equilibrium scheme, 2 for
 //     the forcing scheme) from the phi field into shared memory; the own
 //     site's 19 f and 19 g into registers; (forcing) M'_ab - delta_ab M'_cc / 2
@@ -320,7 +321,7 @@ inline unsigned blocks3(size_t n) {
 }
 
 template <bool FORCING, class real>
-cudaError_t step3_impl(const StepArgs<real>& a, real* phi_buf, cudaStream_t st) {
+cudaError_t step3_impl(const StepArgs<real>& a, real* phi_buf, cudaStream_t st, const int4* work = nullptr, int ctas = 0) {
     using Lay = Step3Layout<FORCING, real>;
     static bool attr = false;
     if (!attr) {
@@ -333,14 +334,16 @@ cudaError_t step3_impl(const StepArgs<real>& a, real* phi_buf, cudaStream_t st) 
     binary_phi_kernel<real><<<blocks3(n), 256, 0, st>>>(a.src, a.pitch, n, phi_buf);
     StepArgs<real> b = a;
     b.phi = phi_buf;
+    if constexpr (sizeof(real) == 4)
+        if (work) return binary_march3(FORCING, b, work, ctas, st);
     const dim3 grid((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY, (a.nz + Lay::BZ - 1) / Lay::BZ);
     binary_step_kernel3<FORCING, real><<<grid, Lay::NT, Lay::BYTES, st>>>(b);
     return cudaGetLastError();
 }
 }  // namespace
 
-cudaError_t binary_step3(bool forcing, const StepArgs<float>& a, float* phi, cudaStream_t st) {
-    return forcing ? step3_impl<true>(a, phi, st) : step3_impl<false>(a, phi, st);
+cudaError_t binary_step3(bool forcing, const StepArgs<float>& a, float* phi, cudaStream_t st, const int4* work, int ctas) {
+    return forcing ? step3_impl<true>(a, phi, st, work, ctas) : step3_impl<false>(a, phi, st, work, ctas);
 }
 cudaError_t binary_step3(bool forcing, const StepArgs<double>& a, double* phi, cudaStream_t st) {
     return forcing ? step3_impl<true>(a, phi, st) : step3_impl<false>(a, phi, st);
