@@ -72,9 +72,15 @@ __global__ void __launch_bounds__(TX* TY) batch_step_kernel(BatchState bs, char*
 }
 
 // The same step with the pair kernel of step2d_pk.cuh ((TX / 2) * TY threads per
-// tile; 32-bit arithmetic): aligned pairs for instances with an even nx.
+// tile; 32-bit arithmetic): aligned pairs for instances with an even nx.  Resident
+// CTAs of 128 threads per SM: nine for 16-bit storage in the forcing scheme (us per
+// step of the 256-instance sweep on a GB300 with 7 / 8 / 9 / 10 / 12: 279 / 286 / 278 /
+// 276 / 283, of its first 24 instances 34.9 / 35.5 / 34.6 / 35.0 / 35.2), else eight
+// (8 / 10 / unbounded: fp16 deviations equilibrium 230 / 234 / 236, float32 280 / 305 /
+// 284 and 256 / 270 / 261).
 template <bool FORCING, class S, int TX, int TY>
-__global__ void __launch_bounds__((TX / 2) * TY) batch_step_kernel_pk(BatchState bs, char* buf, int parity) {
+__global__ void __launch_bounds__((TX / 2) * TY, (FORCING && PairIO<S>::RAW16 ? 1152 : 1024) / ((TX / 2) * TY))
+    batch_step_kernel_pk(BatchState bs, char* buf, int parity) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned count = unsigned(*bs.count);
     for (unsigned item = blockIdx.x; item < count; item += gridDim.x) {

@@ -81,7 +81,7 @@ struct BatchLaunch {
 // The pair kernel (32-bit arithmetic) on the same tiles: (TX / 2) * TY threads.
 template <bool F, class S, int TX, int TY>
 struct BatchLaunchPK : BatchLaunch<F, S, TX, TY> {
-    using Lay = Layout2PK<F, TX, TY>;
+    using Lay = Layout2PK<F, TX, TY, PairIO<S>::RAW16 ? 3 : 2>;
     static void step(const BatchState& bs, char* buf, int parity, int nblocks, cudaStream_t st) {
         batch_step_kernel_pk<F, S, TX, TY><<<nblocks, Lay::NTH, Lay::BYTES, st>>>(bs, buf, parity);
     }

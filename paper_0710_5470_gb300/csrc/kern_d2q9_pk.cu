@@ -11,7 +11,7 @@ namespace {
 
 template <bool F, class S, int TX, int TY>
 struct PK2Launch {
-    using Lay = Layout2PK<F, TX, TY>;
+    using Lay = Layout2PK<F, TX, TY, PairIO<S>::RAW16 ? 3 : 2>;
     static const void* fn() { return reinterpret_cast<const void*>(step_kernel2d_pk<F, S, TX, TY>); }
     static cudaError_t step(const StepArgs& a, dim3 grid, cudaStream_t st) {
         static int attr_done = 0;

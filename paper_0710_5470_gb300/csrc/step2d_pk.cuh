@@ -27,7 +27,7 @@
 
 namespace lbk {
 
-template <bool FORCING, int TX, int TY>
+template <bool FORCING, int TX, int TY, int NMP = 3>
 struct Layout2PK {
     static constexpr int H = FORCING ? 2 : 1;       // density halo in y
     static constexpr int HX = 2;                    // density halo in x (pairs start on even x)
@@ -41,12 +41,12 @@ struct Layout2PK {
     static constexpr int NBR = (NRING + NTH - 1) / NTH;
     static constexpr size_t OFF_RHO = 0;
     static constexpr size_t OFF_MP = (size_t(RN) * 4 + 15) / 16 * 16;
-    static constexpr size_t BYTES = FORCING ? OFF_MP + size_t(SN) * 16 : OFF_MP;
+    static constexpr size_t BYTES = FORCING ? OFF_MP + size_t(SN) * 4 * NMP : OFF_MP;
     static_assert(TX % 4 == 0, "tile width");
     static_assert(NAH <= 2 && NBR <= 2, "items per thread");
-    // M' (Mxx, Myy, Mxy) of ring site (sx, sy): even and odd columns in separate
-    // halves, so that the pair neighbourhoods of consecutive threads are conflict-free
-    __host__ __device__ static constexpr int mp_index(int sx, int sy) { return (sx & 1) * (SY * SXH) + sy * SXH + (sx >> 1); }
+    // NMP components of M' at ring site (sx, sy): one field each, rows of SX (even), so
+    // that the columns of a pair's neighbourhood are two aligned 2-vectors
+    __host__ __device__ static constexpr int mp_index(int sx, int sy) { return sy * SX + sx; }
 };
 
 // Raw word of population i >= 1 of the two sites qa, qb (odd nx: not one aligned pair).
@@ -250,11 +250,14 @@ __device__ __forceinline__ void step2d_pair_tile(const Tile2DArgs& args, int x0,
     using L = D2Q9;
     using IO = PairIO<S>;
     using Wd = typename IO::W;
-    using Lay = Layout2PK<FORCING, TX, TY>;
+    using Lay = Layout2PK<FORCING, TX, TY, IO::RAW16 ? 3 : 2>;
     constexpr int H = Lay::H, HX = Lay::HX, TXP = Lay::TXP, NTH = Lay::NTH;
     constexpr int RX = Lay::RX, RXP = Lay::RXP, SX = Lay::SX;
     float* rho_s = reinterpret_cast<float*>(smem + Lay::OFF_RHO);
-    float4* mp_s = reinterpret_cast<float4*>(smem + Lay::OFF_MP);
+    // 16-bit storage: M'_xx, M'_xy, M'_yy; float32: M'_xx and M'_xy over 12
+    float* mx_s = reinterpret_cast<float*>(smem + Lay::OFF_MP);
+    float* mo_s = mx_s + Lay::SN;
+    float* my_s = mo_s + Lay::SN;
 
     const int nx = args.nx, ny = args.ny;
 #ifdef LB_DEBUG_BOUNDS
@@ -334,9 +337,16 @@ __device__ __forceinline__ void step2d_pair_tile(const Tile2DArgs& args, int x0,
     P2 g[2] = {pp(0.f), pp(0.f)};
     if constexpr (FORCING) {
         auto put_mp = [&](int k, float gx, float gy) {
-            const float hk = 0.5f * pk * (gx * gx + gy * gy);
             LB_GUARD(k >= 0 && k < Lay::SN, BK_2D_SHARED, k, return)
-            mp_s[k] = make_float4(pk * gx * gx - hk, pk * gy * gy - hk, pk * gx * gy, 0.0f);
+            if constexpr (IO::RAW16) {
+                const float hk = 0.5f * pk * (gx * gx + gy * gy);
+                mx_s[k] = pk * gx * gx - hk;
+                my_s[k] = pk * gy * gy - hk;
+                mo_s[k] = pk * gx * gy;
+            } else {
+                mx_s[k] = (pk * (1.0f / 24.0f)) * (gx * gx - gy * gy);
+                mo_s[k] = (pk * (1.0f / 12.0f)) * (gx * gy);
+            }
         };
         put_mp(Lay::mp_index(2 * px + 1, py + 1), G[0].v.x, G[1].v.x);
         put_mp(Lay::mp_index(2 * px + 2, py + 1), G[0].v.y, G[1].v.y);
@@ -359,29 +369,56 @@ __device__ __forceinline__ void step2d_pair_tile(const Tile2DArgs& args, int x0,
             }
         }
         __syncthreads();
-        // g_a = -sum_i w_i sum_b e_ib M'_ab(r + e_i) (Eq. 28): neighbourhood columns
-        // c = 0..3 (sites x-1 .. x+2) and rows -1, 0, +1 of the ring frame
-        float gs[2][2] = {};
+        // Eq. 28 over the columns A = (x - 1, x) and B = (x + 1, x + 2) of the pair
+        auto cols = [&](const float* f, int r, int half) {
+            return P2{*reinterpret_cast<const float2*>(f + Lay::mp_index(2 * px + 2 * half, py + 1 + r))};
+        };
+        if constexpr (IO::RAW16) {
+            // g_a = -sum_i w_i sum_b e_ib M'_ab(r + e_i), neighbours row by row from below
+            // and left to right.  The order is kept: the rounding of 16-bit deviations
+            // amplifies any other, and a batch's instances follow their single runs bit
+            // for bit.  Pairs of columns take 36 shared-memory wavefronts and half the
+            // instructions of site by site with (xx, yy, xy) vectors (48).
+            g[0] = g[1] = pp(0.f);
 #pragma unroll
-        for (int r = -1; r <= 1; ++r) {
+            for (int r = -1; r <= 1; ++r) {
+                const P2 xA = cols(mx_s, r, 0), xB = cols(mx_s, r, 1), oA = cols(mo_s, r, 0), oB = cols(mo_s, r, 1);
+                const P2 yA = cols(my_s, r, 0), yB = cols(my_s, r, 1);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float4 M = mp_s[Lay::mp_index(2 * px + c, py + 1 + r)];
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    const int dx = c - 1 - s;
-                    if (dx < -1 || dx > 1 || (dx == 0 && r == 0)) continue;
+                for (int dx = -1; dx <= 1; ++dx) {
+                    if (r == 0 && dx == 0) continue;
+                    const P2 xx = dx < 0 ? xA : xB, xy = dx < 0 ? oA : (dx > 0 ? oB : pp(oA.v.y, oB.v.x));
+                    const P2 yy = dx < 0 ? yA : (dx > 0 ? yB : pp(yA.v.y, yB.v.x));
+                    // sum_b e_b M'_ab up to the sign of (e_x or else e_y), which goes to the weight
+                    const int sg = dx != 0 ? dx : r;
+                    const P2 ax = dx == 0 ? xy : (r == 0 ? xx : (dx * r > 0 ? xx + xy : xx - xy));
+                    const P2 ay = dx == 0 ? yy : (r == 0 ? xy : (dx * r > 0 ? xy + yy : xy - yy));
                     const float wi = (dx == 0 || r == 0) ? 1.0f / 3.0f : 1.0f / 12.0f;
-                    // sum_b e_b M'_ab: a = x: e_x Mxx + e_y Mxy; a = y: e_x Mxy + e_y Myy
-                    const float ax = float(dx) * M.x + float(r) * M.z;
-                    const float ay = float(dx) * M.z + float(r) * M.y;
-                    gs[s][0] -= wi * ax;
-                    gs[s][1] -= wi * ay;
+                    g[0] = fma(pp(-wi * sg), ax, g[0]);
+                    g[1] = fma(pp(-wi * sg), ay, g[1]);
                 }
             }
+        } else {
+            // g_x = -(d_x D + d_y O), g_y = -(d_x O - d_y D) with D = M'_xx = -M'_yy, O =
+            // M'_xy: per column X f = 4 f_0 + f_+ + f_- and Y f = f_+ - f_- over the rows, 12
+            // d_x f = X(x + 1) - X(x - 1), 12 d_y f = Y(x - 1) + 4 Y(x) + Y(x + 1): 24
+            // instructions and 24 shared-memory wavefronts where three components site by
+            // site took 130 and 48.
+            const P2 four = pp(4.0f);
+            P2 XD[2], YD[2], XO[2], YO[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const P2 dp = cols(mx_s, 1, h), dm = cols(mx_s, -1, h), op = cols(mo_s, 1, h), om = cols(mo_s, -1, h);
+                XD[h] = fma(four, cols(mx_s, 0, h), dp + dm);
+                XO[h] = fma(four, cols(mo_s, 0, h), op + om);
+                YD[h] = dp - dm;
+                YO[h] = op - om;
+            }
+            const P2 yo = fma(four, pp(YO[0].v.y, YO[1].v.x), YO[0] + YO[1]);
+            const P2 yd = fma(four, pp(YD[0].v.y, YD[1].v.x), YD[0] + YD[1]);
+            g[0] = (XD[0] - XD[1]) - yo;
+            g[1] = (XO[0] - XO[1]) + yd;
         }
-        g[0] = pp(gs[0][0], gs[1][0]);
-        g[1] = pp(gs[0][1], gs[1][1]);
     }
 
     // ---------------- stage C: collide and push the own pair
