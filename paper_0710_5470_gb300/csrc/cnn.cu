@@ -195,9 +195,11 @@ __global__ void __launch_bounds__(NTH) conv_tile(const float* in, const __half* 
 // additions of the shares cost more than the sums: 256 CTAs x 9216 of them,
 // 89 us, and 158 us on the 1440 addresses of the first layer.)  Measured (as
 // above): 32 -> 32 channels 42 us against 107 us, 5 -> 32 30 against 42,
-// 32 -> 3 13 against 28.
+// 32 -> 3 13 against 28.  Two CTAs per SM, at 128 registers: with one, at 180, eight
+// warps per SM left the shared loads' latency open, and a pass of training (three
+// epochs of these 16 samples with the copies) took 1558 us against 1500.
 template <int CI, int CO, int OT, int RS>
-__global__ void __launch_bounds__(NTH) conv_bwd_weight(const float* h, const float* dout, float* part, int N, int H, int Wd) {
+__global__ void __launch_bounds__(NTH, 2) conv_bwd_weight(const float* h, const float* dout, float* part, int N, int H, int Wd) {
     constexpr int COP = (CO + 3) / 4 * 4, OG = COP / OT, PL = PLANE + 4, GP = COP == 32 ? COP + 4 : COP;
     static_assert(CI * OG * RS <= NTH && COP % OT == 0 && OT % 4 == 0 && NTH % COP == 0, "work split");
     extern __shared__ __align__(16) float sm[];
