@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(NTH) conv_tile(const float* in, const __half* 
 // 89 us, and 158 us on the 1440 addresses of the first layer.)  Measured (as
 // above): 32 -> 32 channels 42 us against 107 us, 5 -> 32 30 against 42,
 // 32 -> 3 13 against 28.  Two CTAs per SM, at 128 registers: with one, at 180, eight
-// warps per SM left the shared loads' latency open, and a pass of training (three
+// warps per SM left the shared loads' latency open, and a pass of training (four
 // epochs of these 16 samples with the copies) took 1558 us against 1500.
 template <int CI, int CO, int OT, int RS>
 __global__ void __launch_bounds__(NTH, 2) conv_bwd_weight(const float* h, const float* dout, float* part, int N, int H, int Wd) {

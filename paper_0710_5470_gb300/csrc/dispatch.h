@@ -10,6 +10,7 @@ struct LbKernelSet {
     int threads = 0;              // threads per CTA of the fused step
     size_t smem = 0;              // dynamic shared memory of the fused step
     const char* name = "";        // kernel form (reported by lb_kernel_info)
+    int march_warps = 0;          // > 0: D2Q9 marching strips, so many warps per CTA; ty: rows of a chunk
     bool aos = false;             // `step` needs the interleaved 16-bit layout (PopPtrs aos = 1)
     const void* step_fn = nullptr;
     cudaError_t (*step)(const lbk::StepArgs&, dim3 grid, cudaStream_t) = nullptr;

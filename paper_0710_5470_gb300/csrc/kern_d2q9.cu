@@ -54,10 +54,11 @@ static LbKernelSet pick(int storage, int nx, int ny, int sms) {
     return LbKernelSet{};
 }
 
-LbKernelSet lbk_pk2d(int scheme, int storage, LbKernelSet k);
+LbKernelSet lbk_pk2d(int scheme, int storage, LbKernelSet k, int nx, int ny, int sms);
 
 LbKernelSet lbk_kernels_d2q9(int scheme, int storage, int nx, int ny, int sms) {
-    return lbk_pk2d(scheme, storage, scheme == 1 ? pick<true>(storage, nx, ny, sms) : pick<false>(storage, nx, ny, sms));
+    return lbk_pk2d(scheme, storage, scheme == 1 ? pick<true>(storage, nx, ny, sms) : pick<false>(storage, nx, ny, sms),
+                    nx, ny, sms);
 }
 
 // First recorded index violation of this unit's kernels (checked builds; see bounds.cuh).

@@ -1,9 +1,10 @@
 // Instantiations of the two-sites-per-thread D2Q9 step (step2d_pk.cuh) for
 // single lattices.
+#include <algorithm>
 #include <cstdlib>
 
 #include "dispatch.h"
-#include "step2d_pk.cuh"
+#include "step2d_march.cuh"
 
 using namespace lbk;
 
@@ -37,6 +38,30 @@ struct PK2Launch {
     }
 };
 
+// The marching form (step2d_march.cuh): equilibrium scheme, 16-bit storage, even nx.
+template <class S>
+struct MarchLaunch {
+    static const void* fn() { return reinterpret_cast<const void*>(step_kernel2d_march<S>); }
+    static cudaError_t step(const StepArgs& a, dim3 grid, cudaStream_t st) {   // a.lz: rows of a chunk
+        Tile2DArgs t{a.src_base, a.dst_base, a.pitch, a.nx, a.ny, a.pair2d, a.a, a.b, a.T, a.kappa, a.omega,
+                     a.nu, a.fa, a.fb, a.fT, a.fkappa, a.fomega, a.fnu, a.pref, a.rsum, a.status};
+        const int strips = (a.nx + MARCH_COLS - 1) / MARCH_COLS, chunks = (a.ny + a.lz - 1) / a.lz;
+        step_kernel2d_march<S><<<grid, 32 * MARCH_WARPS, 0, st>>>(t, strips, a.lz, strips * chunks);
+        return cudaGetLastError();
+    }
+    static LbKernelSet make(LbKernelSet k, int rows) {
+        k.tx = MARCH_COLS;
+        k.ty = rows;
+        k.threads = 32 * MARCH_WARPS;
+        k.smem = 0;
+        k.step_fn = fn();
+        k.step = &step;
+        k.march_warps = MARCH_WARPS;
+        k.name = "pairs, marching strips of 60 columns, mixed adds";
+        return k;
+    }
+};
+
 template <bool F>
 LbKernelSet pick(int storage, LbKernelSet k) {
     switch (storage) {
@@ -50,12 +75,39 @@ LbKernelSet pick(int storage, LbKernelSet k) {
 
 }  // namespace
 
+// Rows of a marching warp's chunk, 0: the lattice keeps the tiles (LB_D2_ROWS=n
+// forces n, for comparisons).  Resident warps (sixteen per SM) pass through rows + 2
+// rows and about two more in filling and draining; the chunk with the fewest rows in
+// all waves is taken: 2048^2 30 rows (one wave of 2415 warps) 38.5 us, 28 rows (two
+// waves) 47.3, 32 rows 40.5, 40 rows 40.4.  From 8,500 sites per SM on, where a wave of a
+// dozen rows and more fills the chip, tiles -> strips: 1200 x 1100 15.2 -> 14.7, 700 x 2000
+// 16.4 -> 14.8, 1100 x 1400 17.6 -> 16.2; 1024^2 (6900 per SM) 12.5 -> 12.7, 800^2 8.7 -> 10.3.
+int march_rows(int nx, int ny, int sms) {
+    if (const char* e = std::getenv("LB_D2_ROWS")) return std::min(ny, std::max(0, std::atoi(e)));
+    if (nx % 2 != 0 || double(nx) * ny < 8.5e3 * sms) return 0;
+    const long long strips = (nx + MARCH_COLS - 1) / MARCH_COLS, slots = 16LL * std::max(sms, 1);
+    int best = 0;
+    long long cost = 0;
+    for (int r = 12; r <= 64 && r <= ny; ++r) {
+        const long long waves = (strips * ((ny + r - 1) / r) + slots - 1) / slots, c = waves * (r + 4);
+        if (best == 0 || c < cost) {
+            best = r;
+            cost = c;
+        }
+    }
+    return best;
+}
+
 // The pair kernel for D2Q9 with 32-bit arithmetic (storage 1, 2, 3) in place
 // of `step` of `base` (float64 keeps the tile kernel: its arithmetic bounds
 // it).  LB_D2_VARIANT=0 keeps the tile kernel for comparisons.
-LbKernelSet lbk_pk2d(int scheme, int storage, LbKernelSet k) {
+LbKernelSet lbk_pk2d(int scheme, int storage, LbKernelSet k, int nx, int ny, int sms) {
     const char* env = std::getenv("LB_D2_VARIANT");
     if (env && std::atoi(env) == 0) return k;
+    if (scheme != 1 && (storage == 2 || storage == 3) && nx % 2 == 0 && !std::getenv("LB_NO_PAIR")) {
+        const int rows = march_rows(nx, ny, sms);
+        if (rows > 0) return storage == 2 ? MarchLaunch<StF16>::make(k, rows) : MarchLaunch<StBF16>::make(k, rows);
+    }
     return scheme == 1 ? pick<true>(storage, k) : pick<false>(storage, k);
 }
 

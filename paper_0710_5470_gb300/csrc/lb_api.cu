@@ -615,6 +615,10 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
         const int gy = (p->ny + c->ks.ty - 1) / c->ks.ty;
         c->lz = 1;
         c->grid = dim3(gx, gy, 1);
+        if (c->ks.march_warps > 0) {
+            c->lz = c->ks.ty;
+            c->grid = dim3(unsigned(((long long)gx * gy + c->ks.march_warps - 1) / c->ks.march_warps), 1, 1);
+        }
         if (c->D == 3) {
             const std::vector<int4> work = build_work_list(sms, occ, p->nx, p->ny, p->nz, c->ks.tx, c->ks.ty);
             c->lz = work.front().w - work.front().z;
