@@ -7,6 +7,7 @@
 // finalize kernel retires converged or unstable instances and rebuilds the
 // work list on the device.  No kernel waits on another CTA.
 #pragma once
+#include "chain.cuh"
 #include "aux_kernels.cuh"
 #include "step2d_f64.cuh"
 #include "step2d_pk.cuh"
@@ -51,6 +52,7 @@ struct BatchState {
 // launches no CTAs that only find nothing to do.
 template <bool FORCING, class S, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY) batch_step_kernel(BatchState bs, char* buf, int parity) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned count = unsigned(*bs.count);
     for (unsigned item = blockIdx.x; item < count; item += gridDim.x) {
@@ -81,6 +83,7 @@ __global__ void __launch_bounds__(TX* TY) batch_step_kernel(BatchState bs, char*
 template <bool FORCING, class S, int TX, int TY>
 __global__ void __launch_bounds__((TX / 2) * TY, (FORCING && PairIO<S>::RAW16 ? 1152 : 1024) / ((TX / 2) * TY))
     batch_step_kernel_pk(BatchState bs, char* buf, int parity) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned count = unsigned(*bs.count);
     for (unsigned item = blockIdx.x; item < count; item += gridDim.x) {

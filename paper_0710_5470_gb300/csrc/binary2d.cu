@@ -29,6 +29,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "../../include/lb.h"
 #include "binary_common.cuh"
 #include "binary_launch.h"
@@ -60,6 +61,7 @@ __device__ __forceinline__ real laplacian(const real* p, int c) {
 
 template <bool FORCING, class real>
 __global__ void __launch_bounds__(NT) binary_step_kernel(const StepArgs<real> a) {
+    lbk::chain_begin();
     constexpr int H = FORCING ? 2 : 1;
     constexpr int RX = TX + 2 * H, RY = TY + 2 * H, RN = RX * RY;
     constexpr int SX = TX + 2, SY = TY + 2, SN = SX * SY;
@@ -249,6 +251,7 @@ __device__ __forceinline__ void pair_stencil(const float (&c)[3][4], P2& gx, P2&
 
 template <bool FORCING, int MINB, bool F16 = false>
 __global__ void __launch_bounds__(PNT, MINB) binary_step_kernel_pair(const StepArgs<float> a) {
+    lbk::chain_begin();
     constexpr int H = FORCING ? 2 : 1, HX = 2;
     constexpr int RX = PTX_ + 2 * HX, RY = PTY + 2 * H, RN = RX * RY, RXP = RX / 2;
     constexpr int SX = PTX_ + 2, SY = PTY + 2, SN = SX * SY;
@@ -686,19 +689,17 @@ cudaError_t launch_step(lb_binary* c, int from, cudaStream_t st) {
         if (c->pair) {   // float32 or 16-bit, even nx: two sites per thread
             const dim3 grid((c->p.nx + PTX_ - 1) / PTX_, (c->p.ny + PTY - 1) / PTY);
             if (c->f16) {
-                if (forcing) binary_step_kernel_pair<true, PAIR_MINB16, true><<<grid, PNT, 0, st>>>(a);
-                else binary_step_kernel_pair<false, PAIR_MINB16, true><<<grid, PNT, 0, st>>>(a);
-            } else {
-                if (forcing) binary_step_kernel_pair<true, PAIR_MINB><<<grid, PNT, 0, st>>>(a);
-                else binary_step_kernel_pair<false, PAIR_MINB><<<grid, PNT, 0, st>>>(a);
+                return lbk::launch_chained(forcing ? binary_step_kernel_pair<true, PAIR_MINB16, true>
+                                              : binary_step_kernel_pair<false, PAIR_MINB16, true>,
+                                      grid, PNT, 0, st, a);
             }
-            return cudaGetLastError();
+            return lbk::launch_chained(
+                forcing ? binary_step_kernel_pair<true, PAIR_MINB> : binary_step_kernel_pair<false, PAIR_MINB>, grid,
+                PNT, 0, st, a);
         }
     }
     const dim3 grid((c->p.nx + TX - 1) / TX, (c->p.ny + TY - 1) / TY);
-    if (forcing) binary_step_kernel<true, real><<<grid, NT, 0, st>>>(a);
-    else binary_step_kernel<false, real><<<grid, NT, 0, st>>>(a);
-    return cudaGetLastError();
+    return lbk::launch_chained(forcing ? binary_step_kernel<true, real> : binary_step_kernel<false, real>, grid, NT, 0, st, a);
 }
 
 cudaError_t step_once(lb_binary* c, int from, cudaStream_t st) {
@@ -812,8 +813,8 @@ bool is_fin(double v) { return std::isfinite(v); }
 
 // Whether a float32 D3Q19 lattice runs the marching step (LB_B3_MARCH=0 / 1 forces
 // it, for comparisons).  Small lattices give its long CTAs too little to share out:
-// us per step, bricks / march, 32^3 7.2 / 13.3 (forcing) and 5.4 / 10.6 (equilibrium),
-// 48^3 15.7 / 16.3 and 11.3 / 12.7, 64^3 24.4 / 20.9 and 17.4 / 16.4.
+// us per step, bricks / march, 32^3 6.8 / 13.2 (forcing) and 4.8 / 10.2 (equilibrium),
+// 48^3 15.3 / 14.9 and 10.9 / 11.5, 64^3 24.3 / 19.7 and 17.2 / 15.7.
 bool march3_wanted(long long sites) {
     if (const char* e = std::getenv("LB_B3_MARCH")) return std::atoi(e) != 0;
     return sites >= 150000;

@@ -22,6 +22,7 @@
 
 #include "binary_common.cuh"
 #include "binary_launch.h"
+#include "chain.cuh"
 
 namespace lbb {
 
@@ -36,6 +37,7 @@ constexpr int brick_z() { return 2; }
 
 template <class real>
 __global__ void binary_phi_kernel(const real* src, unsigned pitch, unsigned n, real* phi) {
+    lbk::chain_begin();
     for (unsigned s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         real p = 0;
 #pragma unroll
@@ -108,6 +110,7 @@ struct Step3Layout {
 template <bool FORCING, class real>
 __global__ void __launch_bounds__(BX * BY * brick_z<real>(), sizeof(real) == 4 ? 3 : 1)
     binary_step_kernel3(const StepArgs<real> a) {
+    lbk::chain_begin();
     using Lay = Step3Layout<FORCING, real>;
     constexpr int H = Lay::H, RX = Lay::RX, RY = Lay::RY, RN = Lay::RN;
     constexpr int SX = Lay::SX, SY = Lay::SY, SN = Lay::SN;
@@ -331,14 +334,14 @@ cudaError_t step3_impl(const StepArgs<real>& a, real* phi_buf, cudaStream_t st, 
         attr = true;
     }
     const unsigned n = unsigned(a.nx) * unsigned(a.ny) * unsigned(a.nz);
-    binary_phi_kernel<real><<<blocks3(n), 256, 0, st>>>(a.src, a.pitch, n, phi_buf);
+    const cudaError_t e = lbk::launch_chained(binary_phi_kernel<real>, blocks3(n), 256, 0, st, a.src, a.pitch, n, phi_buf);
+    if (e != cudaSuccess) return e;
     StepArgs<real> b = a;
     b.phi = phi_buf;
     if constexpr (sizeof(real) == 4)
         if (work) return binary_march3(FORCING, b, work, ctas, st);
     const dim3 grid((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY, (a.nz + Lay::BZ - 1) / Lay::BZ);
-    binary_step_kernel3<FORCING, real><<<grid, Lay::NT, Lay::BYTES, st>>>(b);
-    return cudaGetLastError();
+    return lbk::launch_chained(binary_step_kernel3<FORCING, real>, grid, Lay::NT, Lay::BYTES, st, b);
 }
 }  // namespace
 

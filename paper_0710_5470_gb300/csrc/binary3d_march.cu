@@ -28,8 +28,7 @@ int binary_march3_ctas(bool forcing, int nx) {
 }
 
 cudaError_t binary_march3(bool forcing, const StepArgs<float>& a, const int4* work, int ctas, cudaStream_t st) {
-    kernel(forcing, a.nx)<<<ctas, Lay3::NTH, Lay3::bytes(forcing), st>>>(March3Args{a, work});
-    return cudaGetLastError();
+    return lbk::launch_chained(kernel(forcing, a.nx), ctas, Lay3::NTH, Lay3::bytes(forcing), st, March3Args{a, work});
 }
 
 }  // namespace lbb

@@ -14,14 +14,15 @@
 // forcing scheme, bound by issue; this one has 640 and is bound by the loads of the
 // 38 populations.  Measured on a GB300, us per step with the phi pass (27 us at
 // 128^3), bricks -> march:
-// 64^3 forcing 24.4 -> 20.9, 101 x 75 x 53 45.5 -> 36.3, 128^3 189 -> 147 (388 bytes
-// per site at 82% of the copy bandwidth), 256^3 1459 -> 1272; equilibrium 64^3 17.4
-// -> 16.4, 128^3 152 -> 134, 256^3 1268 -> 1192.
+// 64^3 forcing 24.3 -> 19.7, 101 x 75 x 53 45.4 -> 36.7, 128^3 189 -> 146 (388 bytes
+// per site at 82% of the copy bandwidth), 256^3 1459 -> 1288; equilibrium 64^3 17.2
+// -> 15.7, 128^3 152 -> 131, 256^3 1263 -> 1179 (launches chained).
 //
 // AL: nx even, so that pairs are aligned 2-vectors and never split by the periodic
 // wrap; otherwise every site of a pair is loaded and stored on its own.
 #pragma once
 #include "binary_common.cuh"
+#include "chain.cuh"
 #include "step3d_pk_eq.cuh"
 
 namespace lbb {
@@ -132,6 +133,7 @@ struct Form {
 // four (128 registers, spills) 25%.
 template <bool FORCING, int TX, int TY, bool AL>
 __global__ void __launch_bounds__((TX / 2) * TY, 3) binary_step_kernel3_march(const March3Args args) {
+    lbk::chain_begin();
     using L = D3Q19;
     using Lay = lbk::LayoutPK<TX, TY, true>;
     using LF = LayoutMarch3<TX, TY>;
@@ -200,8 +202,8 @@ __global__ void __launch_bounds__((TX / 2) * TY, 3) binary_step_kernel3_march(co
         for (int m = 0; m < NA; ++m) {
             if (tid + m * NTH < NIT) {
                 const unsigned q = ld_off + a_in[m];
-                if constexpr (AL) rn[m] = __ldg(reinterpret_cast<const float2*>(a.phi) + (q >> 1));
-                else rn[m].x = __ldg(a.phi + q);
+                if constexpr (AL) rn[m] = reinterpret_cast<const float2*>(a.phi)[q >> 1];
+                else rn[m].x = a.phi[q];
             }
         }
         advance(ld_off);
@@ -210,8 +212,8 @@ __global__ void __launch_bounds__((TX / 2) * TY, 3) binary_step_kernel3_march(co
     // population k (f_0..f_18, g_0..g_18) of the own pair of the plane collided next
     auto load = [&](int k) -> P2 {
         const unsigned q = unsigned(k) * pitch + zr[1] + yr[1];
-        if constexpr (AL) return P2{__ldg(reinterpret_cast<const float2*>(src) + ((q + xc) >> 1))};
-        else return pp(__ldg(src + q + xc), __ldg(src + q + xp1));
+        if constexpr (AL) return P2{reinterpret_cast<const float2*>(src)[(q + xc) >> 1]};
+        else return pp(src[q + xc], src[q + xp1]);
     };
 
     lbk::StencilAcc<float> acc{0, 0, 0, 0, 0, 0, 0};

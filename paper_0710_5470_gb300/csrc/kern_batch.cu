@@ -40,7 +40,7 @@ struct BatchLaunch {
     static constexpr size_t BYTES = sizeof(typename S::real) == 8 ? Layout64<F, TX, TY, TX * TY>::BYTES
                                                                    : StepLayout<D2Q9, F, TX, TY, typename S::real>::BYTES;
     static void step(const BatchState& bs, char* buf, int parity, int nblocks, cudaStream_t st) {
-        batch_step_kernel<F, S, TX, TY><<<nblocks, TX * TY, BYTES, st>>>(bs, buf, parity);
+        launch_chained(batch_step_kernel<F, S, TX, TY>, nblocks, TX * TY, BYTES, st, bs, buf, parity);
     }
     static void check(const BatchState& bs, const char* buf, int parity, int nblocks, cudaStream_t st) {
         batch_check_kernel<S, TX, TY><<<nblocks, TX * TY, 0, st>>>(bs, buf, parity);
@@ -83,7 +83,7 @@ template <bool F, class S, int TX, int TY>
 struct BatchLaunchPK : BatchLaunch<F, S, TX, TY> {
     using Lay = Layout2PK<F, TX, TY, PairIO<S>::RAW16 ? 3 : 2>;
     static void step(const BatchState& bs, char* buf, int parity, int nblocks, cudaStream_t st) {
-        batch_step_kernel_pk<F, S, TX, TY><<<nblocks, Lay::NTH, Lay::BYTES, st>>>(bs, buf, parity);
+        launch_chained(batch_step_kernel_pk<F, S, TX, TY>, nblocks, Lay::NTH, Lay::BYTES, st, bs, buf, parity);
     }
     static BatchKernels make() {
         BatchKernels k = BatchLaunch<F, S, TX, TY>::make();

@@ -14,9 +14,8 @@ static LbKernelSet f64_tile(LbKernelSet k) {
     k.smem = Lay::BYTES;
     k.step_fn = reinterpret_cast<const void*>(step_kernel2d_f64<F, TX, TY, NTH>);
     k.step = [](const StepArgs& a, dim3 grid, cudaStream_t st) -> cudaError_t {
-        step_kernel2d_f64<F, TX, TY, NTH><<<grid, NTH, Lay::BYTES, st>>>(
-            tile2d_args(a), consts64(a.a, a.b, a.T, a.kappa, a.omega, a.nu));
-        return cudaGetLastError();
+        return launch_chained(step_kernel2d_f64<F, TX, TY, NTH>, grid, NTH, Lay::BYTES, st, tile2d_args(a),
+                              consts64(a.a, a.b, a.T, a.kappa, a.omega, a.nu));
     };
     return k;
 }

@@ -23,8 +23,7 @@ struct PK2Launch {
         }
         Tile2DArgs t{a.src_base, a.dst_base, a.pitch, a.nx, a.ny, a.pair2d, a.a, a.b, a.T, a.kappa, a.omega,
                      a.nu, a.fa, a.fb, a.fT, a.fkappa, a.fomega, a.fnu, a.pref, a.rsum, a.status};
-        step_kernel2d_pk<F, S, TX, TY><<<grid, Lay::NTH, Lay::BYTES, st>>>(t);
-        return cudaGetLastError();
+        return launch_chained(step_kernel2d_pk<F, S, TX, TY>, grid, Lay::NTH, Lay::BYTES, st, t);
     }
     static void apply(LbKernelSet& k, const char* name) {
         k.tx = TX;
@@ -46,8 +45,7 @@ struct MarchLaunch {
         Tile2DArgs t{a.src_base, a.dst_base, a.pitch, a.nx, a.ny, a.pair2d, a.a, a.b, a.T, a.kappa, a.omega,
                      a.nu, a.fa, a.fb, a.fT, a.fkappa, a.fomega, a.fnu, a.pref, a.rsum, a.status};
         const int strips = (a.nx + MARCH_COLS - 1) / MARCH_COLS, chunks = (a.ny + a.lz - 1) / a.lz;
-        step_kernel2d_march<S><<<grid, 32 * MARCH_WARPS, 0, st>>>(t, strips, a.lz, strips * chunks);
-        return cudaGetLastError();
+        return launch_chained(step_kernel2d_march<S>, grid, 32 * MARCH_WARPS, 0, st, t, strips, a.lz, strips * chunks);
     }
     static LbKernelSet make(LbKernelSet k, int rows) {
         k.tx = MARCH_COLS;

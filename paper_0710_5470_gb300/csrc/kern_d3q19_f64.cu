@@ -21,8 +21,7 @@ cudaError_t run(K kernel, Args64x3 a, int first, int planes, cudaStream_t st) {
     a.first = first;
     a.planes = planes;
     const unsigned n = unsigned(a.nx) * unsigned(a.ny) * unsigned(planes);
-    kernel<<<(n + THREADS - 1) / THREADS, THREADS, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(kernel, (n + THREADS - 1) / THREADS, THREADS, 0, st, a);
 }
 
 template <bool F>

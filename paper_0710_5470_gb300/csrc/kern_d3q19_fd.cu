@@ -16,9 +16,9 @@ struct FDLaunch {
     static const void* fn() { return reinterpret_cast<const void*>(step_kernel3d_fd<S, TX, TY, 3, AOS, AL>); }
     static cudaError_t step(const StepArgs& a, dim3 grid, cudaStream_t st) {
         const unsigned pairs = (unsigned(a.nx) * unsigned(a.ny) * unsigned(a.nz) + 1u) / 2u;
-        density_pairs<S, AOS><<<(pairs + 255u) / 256u, 256, 0, st>>>(a, pairs);
-        step_kernel3d_fd<S, TX, TY, 3, AOS, AL><<<grid, Lay::NTH, Lay::BYTES, st>>>(a);
-        return cudaGetLastError();
+        const cudaError_t e = launch_chained(density_pairs<S, AOS>, (pairs + 255u) / 256u, 256, 0, st, a, pairs);
+        return e != cudaSuccess ? e
+                                : launch_chained(step_kernel3d_fd<S, TX, TY, 3, AOS, AL>, grid, Lay::NTH, Lay::BYTES, st, a);
     }
     static LbKernelSet apply(LbKernelSet k, const char* name) {
         k.tx = TX;

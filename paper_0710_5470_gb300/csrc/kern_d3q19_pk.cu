@@ -19,8 +19,7 @@ struct PKLaunch {
             if (e != cudaSuccess) return e;
             attr_done = 1;
         }
-        step_kernel3d_pk<S, TX, TY, MINB, PF, MIXED, AOS, PB><<<grid, Lay::NTH, Lay::BYTES, st>>>(a);
-        return cudaGetLastError();
+        return launch_chained(step_kernel3d_pk<S, TX, TY, MINB, PF, MIXED, AOS, PB>, grid, Lay::NTH, Lay::BYTES, st, a);
     }
     static void apply(LbKernelSet& k, const char* name) {
         k.tx = TX;

@@ -20,8 +20,7 @@ struct PKELaunch {
             if (e != cudaSuccess) return e;
             attr_done = 1;
         }
-        step_kernel3d_pk_eq<S, TX, TY, MINB, AOS><<<grid, Lay::NTH, Lay::BYTES, st>>>(a);
-        return cudaGetLastError();
+        return launch_chained(step_kernel3d_pk_eq<S, TX, TY, MINB, AOS>, grid, Lay::NTH, Lay::BYTES, st, a);
     }
     static void apply(LbKernelSet& k, const char* name) {
         k.tx = TX;

@@ -31,12 +31,12 @@ struct StepKernelOf {
     }
     static void launch(dim3 grid, cudaStream_t st, const StepArgs& a) {
         if constexpr (D3) {
-            step_kernel3d<FORCING, S, TX, TY, PAIR><<<grid, TX * TY, bytes(), st>>>(a);
+            launch_chained(step_kernel3d<FORCING, S, TX, TY, PAIR>, grid, TX * TY, bytes(), st, a);
         } else if constexpr (F64) {
-            step_kernel2d_f64<FORCING, TX, TY, TX * TY><<<grid, TX * TY, bytes(), st>>>(
-                tile2d_args(a), consts64(a.a, a.b, a.T, a.kappa, a.omega, a.nu));
+            launch_chained(step_kernel2d_f64<FORCING, TX, TY, TX * TY>, grid, TX * TY, bytes(), st, tile2d_args(a),
+                           consts64(a.a, a.b, a.T, a.kappa, a.omega, a.nu));
         } else {
-            step_kernel<L, FORCING, S, TX, TY><<<grid, TX * TY, bytes(), st>>>(tile2d_args(a));
+            launch_chained(step_kernel<L, FORCING, S, TX, TY>, grid, TX * TY, bytes(), st, tile2d_args(a));
         }
     }
 };

@@ -20,6 +20,7 @@
 // 315 -> 236 (3.6 G sites/s; with 155 operations per site, halo included, 90% of
 // the FP64 pipe).
 #pragma once
+#include "chain.cuh"
 #include "step_kernel.cuh"
 
 namespace lbk {
@@ -251,6 +252,7 @@ __device__ __forceinline__ void step2d_tile_f64(const Tile2DArgs& args, const Co
 // One step of a single D2Q9 lattice: one CTA per tile.
 template <bool FORCING, int TX, int TY, int NTH>
 __global__ void __launch_bounds__(NTH) step_kernel2d_f64(const Tile2DArgs args, const Consts64 k) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     step2d_tile_f64<FORCING, TX, TY, NTH>(args, k, blockIdx.x * TX, blockIdx.y * TY, reinterpret_cast<double*>(smem_raw));
 }

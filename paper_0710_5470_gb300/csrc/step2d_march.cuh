@@ -19,6 +19,7 @@
 // 12.5 -> 12.7.  Rows in flight 1 / 2 / 3 at 2048^2 and 32 rows: 41.3 / 40.5 / 50 (168
 // registers).
 #pragma once
+#include "chain.cuh"
 #include "step2d_pk.cuh"
 
 namespace lbk {
@@ -152,6 +153,7 @@ __device__ __forceinline__ void step2d_march(const Tile2DArgs& args, int x0, int
 template <class S>
 __global__ void __launch_bounds__(32 * MARCH_WARPS, 4) step_kernel2d_march(const Tile2DArgs args, int strips, int rows,
                                                                           int items) {
+    chain_begin();
     const int item = blockIdx.x * MARCH_WARPS + threadIdx.x / 32;
     if (item >= items) return;
     const int x0 = (item % strips) * MARCH_COLS, y0 = (item / strips) * rows;

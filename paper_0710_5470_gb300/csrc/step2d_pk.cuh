@@ -21,6 +21,7 @@
 // pair is loaded and stored on its own, wrapped on its own, and a pair whose
 // second site lies beyond the lattice stores its first site only.
 #pragma once
+#include "chain.cuh"
 #include "bounds.cuh"
 #include "step3d_pk.cuh"
 #include "step_kernel.cuh"
@@ -476,6 +477,7 @@ __device__ __forceinline__ void step2d_pair_tile(const Tile2DArgs& args, int x0,
 template <bool FORCING, class S, int TX, int TY>
 __global__ void __launch_bounds__((TX / 2) * TY, (PairIO<S>::RAW16 ? 1280 : 1024) / ((TX / 2) * TY))
     step_kernel2d_pk(const Tile2DArgs args) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (args.pair) step2d_pair_tile<FORCING, S, TX, TY, true>(args, blockIdx.x * TX, blockIdx.y * TY, smem_raw);
     else step2d_pair_tile<FORCING, S, TX, TY, false>(args, blockIdx.x * TX, blockIdx.y * TY, smem_raw);

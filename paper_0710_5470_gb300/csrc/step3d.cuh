@@ -21,6 +21,7 @@
 #pragma once
 #include <type_traits>
 
+#include "chain.cuh"
 #include "bounds.cuh"
 #include "step_kernel.cuh"
 
@@ -157,6 +158,7 @@ __device__ __forceinline__ void start(StencilAcc<real>& a, const PlaneParts<real
 // (requires an even nx); otherwise one site per thread.
 template <bool FORCING, class S, int TX, int TY, bool PAIR>
 __global__ void __launch_bounds__(TX* TY, (sizeof(typename S::real) == 4 && TX * TY <= 256) ? 2 : 1) step_kernel3d(const StepArgs args) {
+    chain_begin();
     using L = D3Q19;
     using real = typename S::real;
     constexpr bool RAW = sizeof(typename S::rawi) == 2;

@@ -21,6 +21,7 @@
 // fits its limit, else slabs of planes with two (forcing) or one halo planes on
 // either side, computed one slab after the other (kern_d3q19_f64.cu).
 #pragma once
+#include "chain.cuh"
 #include "bounds.cuh"
 #include "step_kernel.cuh"
 
@@ -99,6 +100,7 @@ __device__ __forceinline__ double density19_f64(const double (&f)[19]) {
 }
 
 __global__ void __launch_bounds__(THREADS64) density3_f64(const Args64x3 a) {
+    chain_begin();
     Site3 s;
     if (!site3(a, s)) return;
     const size_t q = (size_t(s.z) * a.ny + s.y) * a.nx + s.x;
@@ -135,6 +137,7 @@ __device__ __forceinline__ void stencil19_f64(const double* rho, const Site3& s,
 }
 
 __global__ void __launch_bounds__(THREADS64) mprime3_f64(const Args64x3 a) {
+    chain_begin();
     Site3 s;
     if (!site3(a, s)) return;
     const unsigned at = s.at(0, 0, 0);
@@ -305,6 +308,7 @@ __device__ __forceinline__ void collide19_f64(const double (&f)[19], double rho,
 
 template <bool FORCING>
 __global__ void __launch_bounds__(THREADS64, 16) collide3_f64(const Args64x3 a) {
+    chain_begin();
     using L = D3Q19;
     Site3 s;
     if (!site3(a, s)) return;

@@ -25,6 +25,7 @@
 // its own, wrapped on its own, and a pair whose second site lies beyond the
 // lattice stores its first site only.
 #pragma once
+#include "chain.cuh"
 #include "step2d_pk.cuh"   // ld_split
 #include "step3d_pk.cuh"
 
@@ -34,6 +35,7 @@ namespace lbk {
 // sites, whatever its shape (the arrays are padded to whole 128-site rows).
 template <class S, bool AOS>
 __global__ void __launch_bounds__(256) density_pairs(const StepArgs a, unsigned pairs) {
+    chain_begin();
     using IO = PairIO<S>;
     const unsigned t = blockIdx.x * 256u + threadIdx.x;
     if (t >= pairs) return;
@@ -64,6 +66,7 @@ struct LayoutFD {
 
 template <class S, int TX, int TY, int MINB, bool AOS, bool AL>
 __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const StepArgs args) {
+    chain_begin();
     using L = D3Q19;
     using IO = PairIO<S>;
     using Wd = typename IO::W;

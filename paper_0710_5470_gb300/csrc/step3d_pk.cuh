@@ -26,6 +26,7 @@
 // Two barriers per plane: after stage A (densities of the plane visible) and
 // after stage B (M' of the plane visible).
 #pragma once
+#include "chain.cuh"
 #include "bounds.cuh"
 #include "step3d.cuh"
 
@@ -482,6 +483,7 @@ __host__ __device__ __forceinline__ unsigned aos_bytes(unsigned q) {
 // pair with the paired stencils (plane_parts2) instead of site by site.
 template <class S, int TX, int TY, int MINB, int PF, bool MIXED, bool AOS = false, bool PB = false>
 __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk(const StepArgs args) {
+    chain_begin();
     using L = D3Q19;
     using IO = PairIO<S>;
     using Wd = typename IO::W;

@@ -13,6 +13,7 @@
 // collision of plane p - 1 follows the density of plane p directly: a density
 // halo of one row in y, two stash slots, one barrier per plane.
 #pragma once
+#include "chain.cuh"
 #include "step3d_pk.cuh"
 
 namespace lbk {
@@ -134,6 +135,7 @@ struct PairCollEq {
 
 template <class S, int TX, int TY, int MINB, bool AOS>
 __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk_eq(const StepArgs args) {
+    chain_begin();
     using L = D3Q19;
     using IO = PairIO<S>;
     using Wd = typename IO::W;

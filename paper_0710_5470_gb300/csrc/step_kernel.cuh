@@ -26,6 +26,7 @@
 // expanded at compile time (static_for), so velocity components and weights
 // are literals in the generated code.
 #pragma once
+#include "chain.cuh"
 #include "lattice.cuh"
 #include "storage.cuh"
 #include "bounds.cuh"
@@ -568,6 +569,7 @@ __device__ __forceinline__ void step2d_tile(const Tile2DArgs& args, int x0, int 
 // One step of a single D2Q9 lattice: one CTA per tile.
 template <class L, bool FORCING, class S, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY) step_kernel(const Tile2DArgs args) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     step2d_tile<L, FORCING, S, TX, TY>(args, blockIdx.x * TX, blockIdx.y * TY,
                                        reinterpret_cast<typename S::real*>(smem_raw));
