@@ -74,20 +74,23 @@ LbKernelSet pick(int storage, LbKernelSet k) {
 }  // namespace
 
 // Rows of a marching warp's chunk, 0: the lattice keeps the tiles (LB_D2_ROWS=n
-// forces n, for comparisons).  Resident warps (sixteen per SM) pass through rows + 2
-// rows and about two more in filling and draining; the chunk with the fewest rows in
-// all waves is taken: 2048^2 30 rows (one wave of 2415 warps) 38.5 us, 28 rows (two
-// waves) 47.3, 32 rows 40.5, 40 rows 40.4.  From 8,500 sites per SM on, where a wave of a
-// dozen rows and more fills the chip, tiles -> strips: 1200 x 1100 15.2 -> 14.7, 700 x 2000
-// 16.4 -> 14.8, 1100 x 1400 17.6 -> 16.2; 1024^2 (6900 per SM) 12.5 -> 12.7, 800^2 8.7 -> 10.3.
+// forces n, for comparisons).  A warp passes through rows + 2 rows and about two more in
+// filling and draining, each in a time of 1.2 + its SM's CTAs, of which four are
+// resident (12 rows: 12.4 us with up to three per SM, 15.3 with four; 14 rows 14.0 and
+// 17.4); the rows with the least time over all waves are taken: 2048^2 30 rows (one wave of
+// 604 CTAs) 37.6 us, 28 rows (two waves) 46.2, 32 rows 39.5, 40 rows 39.4.  From 7,200 sites
+// per SM on, where a wave of a dozen rows and more fills the chip, tiles -> strips, chained
+// launches: 1100^2 13.8 -> 12.5, 1200 x 1100 14.6 -> 13.3, 700 x 2000 15.7 -> 14.1, 3000 x 400
+// 13.4 -> 12.4, 1500 x 1400 22.4 -> 18.6; 1024^2 (6,900 per SM) 11.8 -> 12.4, 800^2 8.1 -> 9.5.
 int march_rows(int nx, int ny, int sms) {
     if (const char* e = std::getenv("LB_D2_ROWS")) return std::min(ny, std::max(0, std::atoi(e)));
-    if (nx % 2 != 0 || double(nx) * ny < 8.5e3 * sms) return 0;
-    const long long strips = (nx + MARCH_COLS - 1) / MARCH_COLS, slots = 16LL * std::max(sms, 1);
+    if (nx % 2 != 0 || double(nx) * ny < 7.2e3 * sms) return 0;
+    const long long strips = (nx + MARCH_COLS - 1) / MARCH_COLS;
     int best = 0;
-    long long cost = 0;
+    double cost = 0;
     for (int r = 12; r <= 64 && r <= ny; ++r) {
-        const long long waves = (strips * ((ny + r - 1) / r) + slots - 1) / slots, c = waves * (r + 4);
+        const long long ctas = (strips * ((ny + r - 1) / r) + MARCH_WARPS - 1) / MARCH_WARPS, last = ctas % (4LL * sms);
+        const double c = (r + 4) * (5.2 * double(ctas / (4LL * sms)) + (last ? 1.2 + double((last + sms - 1) / sms) : 0.0));
         if (best == 0 || c < cost) {
             best = r;
             cost = c;

@@ -47,22 +47,24 @@ LbKernelSet pick(int nx, LbKernelSet k) {
 // Whether a lattice runs the two-pass form (LB_D3_FIELD=0 / 1 forces it, for
 // comparisons).  us per step on a GB300, fused -> two passes:
 //   float32, even nx: the fused kernel holds two CTAs per SM (82 KB of shared
-//     memory).  48^3 11.8 -> 12.5 (the second launch), 64^3 17.2 -> 15.9, 96^3
-//     44.1 -> 35.1, 128^3 93.4 -> 82.6, 256^3 729 -> 675, 320^3 1347 -> 1294, 384^3
-//     2342 -> 2409 (HBM);
-//   odd nx: the fused form is the one-site tile kernel.  fp16 deviations 33 x 40 x
-//     25 17.4 -> 16.3, 101 x 75 x 53 30.7 -> 26.3, 97 x 101 x 103 63.3 -> 51.0, 201 x
-//     190 x 180 348 -> 347; float32 17.3 -> 14.4, 31.9 -> 25.2, 71.8 -> 55.1, 372 -> 385;
-//   16-bit, even nx, one array per population: 24^3 12.9 -> 11.8, 100 x 76 x 54
-//     25.3 -> 23.4, 200 x 190 x 180 252 -> 232;
-//   16-bit, interleaved blocks: 64^3 16.1 -> 15.7, 96^3 34.0 -> 30.7, then even:
-//     128^3 66.4 -> 66.8 (both buffers no longer fit the L2), 512^3 3570 -> 3585.
+//     memory).  16^3 9.5 -> 8.7, 32^3 10.3 -> 9.6, 48^3 10.9 -> 10.4, 64^3 15.8 ->
+//     13.7, 96^3 42.9 -> 33.0, 128^3 92.2 -> 80.1, 256^3 728 -> 673, 320^3 1345 -> 1290,
+//     384^3 2342 -> 2397 (HBM);
+//   odd nx: the fused form is the one-site tile kernel.  fp16 deviations 9 x 10 x 11
+//     16.9 -> 13.3, 33 x 40 x 25 16.2 -> 13.9, 101 x 75 x 53 29.5 -> 23.7, 97 x 101 x 103
+//     62.2 -> 48.5, 201 x 190 x 180 347 -> 345, 221 x 220 x 210 443 -> 445; float32
+//     16.3 -> 12.7, 16.0 -> 12.0, 30.9 -> 23.4, 70.8 -> 52.9, 371 -> 381;
+//   16-bit, even nx, one array per population: 24^3 11.3 -> 9.1, 100 x 76 x 54
+//     23.9 -> 20.4, 200 x 190 x 180 251 -> 230;
+//   16-bit, interleaved blocks: 32^3 10.3 -> 9.4, 64^3 15.1 -> 13.2, 96^3 32.9 -> 28.6,
+//     then near even: 128^3 65.2 -> 64.1 (both buffers no longer fit the L2), 160 x
+//     160 x 128 99.3 -> 98.5, 512^3 3554 -> 3569.
 bool lbk_fd_wanted(int storage, int nx, size_t sites) {
     if (const char* e = std::getenv("LB_D3_FIELD")) return std::atoi(e) != 0;
     const double n = double(sites);
     if (nx % 2 != 0) return n <= (storage == 1 ? 4e6 : 7e6);
-    if (storage == 1) return n >= 1.5e5 && n <= 4e7;
-    return nx % AOS_SITES != 0 || n <= 1.6e6;
+    if (storage == 1) return n <= 4e7;
+    return nx % AOS_SITES != 0 || n <= 3.4e6;
 }
 
 LbKernelSet lbk_fd_forcing(int storage, int nx, LbKernelSet k) {

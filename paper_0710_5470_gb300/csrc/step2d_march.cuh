@@ -14,9 +14,9 @@
 // on a third: 197 instructions per site against about 330.  A row takes a warp half a
 // microsecond however few there are, so the form is for lattices that fill the chip
 // with chunks of a dozen rows and more (march_rows in kern_d2q9_pk.cu).  Measured on
-// a GB300, us per step, tiles -> strips, fp16 deviations: 2048^2 45.1 -> 38.4 (4.4 TB/s),
-// 4096^2 164.5 -> 138.3 (4.9 TB/s), 1500 x 1400 22.9 -> 19.1, 600 x 5000 33.1 -> 27.5; 1024^2
-// 12.5 -> 12.7.  Rows in flight 1 / 2 / 3 at 2048^2 and 32 rows: 41.3 / 40.5 / 50 (168
+// a GB300, us per step, tiles -> strips, fp16 deviations: 2048^2 44.4 -> 37.6 (4.5 TB/s),
+// 4096^2 164.4 -> 137.6 (4.9 TB/s), 1500 x 1400 22.4 -> 18.6, 600 x 5000 32.6 -> 27.0; 1024^2
+// 11.8 -> 12.4 (chained launches).  Rows in flight 1 / 2 / 3 at 2048^2 and 32 rows: 41.3 / 40.5 / 50 (168
 // registers).
 #pragma once
 #include "chain.cuh"

@@ -36,8 +36,8 @@ def test_both_forms(shape, storage, tol, monkeypatch):
         assert rel_inf(out["1"], O.run(start, m, steps)) < steps * tol
 
 
-@pytest.mark.parametrize("shape,storage,field", [((48, 48, 48), F32, False), ((64, 64, 64), F32, True),
-                                                 ((96, 96, 96), F16DEV, True), ((128, 128, 128), F16DEV, False),
+@pytest.mark.parametrize("shape,storage,field", [((24, 24, 24), F32, True), ((360, 360, 320), F32, False),
+                                                 ((96, 96, 96), F16DEV, True), ((160, 160, 160), F16DEV, False),
                                                  ((100, 20, 10), BF16DEV, True), ((101, 20, 10), F32, True)])
 def test_which_form(shape, storage, field, monkeypatch):
     monkeypatch.delenv("LB_D3_FIELD", raising=False)

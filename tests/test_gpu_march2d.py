@@ -29,7 +29,7 @@ def test_same_bits_as_tiles(shape, storage, monkeypatch):
         assert np.array_equal(got, out[0]), rows
 
 
-@pytest.mark.parametrize("shape,march", [((2048, 2048), True), ((4096, 500), True), ((1024, 1024), False),
+@pytest.mark.parametrize("shape,march", [((2048, 2048), True), ((4096, 500), True), ((1100, 1100), True), ((1024, 1024), False),
                                          ((2047, 2048), False)])
 def test_which_form(shape, march, monkeypatch):
     monkeypatch.delenv("LB_D2_ROWS", raising=False)
