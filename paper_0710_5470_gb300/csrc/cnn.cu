@@ -85,6 +85,7 @@ __device__ __forceinline__ void load_tile(float* tile, const float* in, int x0, 
 template <int CI, int CO, int PX, int OC, bool BACK, bool TANH>
 __global__ void __launch_bounds__(NTH) conv_tile(const float* in, const __half* W, const float* bias, const float* h,
                                                  float* out, int H, int Wd) {
+    lbk::chain_begin();
     constexpr int COP = (CO + 3) / 4 * 4, QW = TILE / PX, NQ = QW * TILE;
     static_assert(NQ * (COP / OC) == NTH && COP % OC == 0 && OC % 4 == 0 && (PX == 4 || PX == 1), "work split");
     extern __shared__ __align__(16) float sm[];
@@ -197,9 +198,11 @@ __global__ void __launch_bounds__(NTH) conv_tile(const float* in, const __half* 
 // above): 32 -> 32 channels 42 us against 107 us, 5 -> 32 30 against 42,
 // 32 -> 3 13 against 28.  Two CTAs per SM, at 128 registers: with one, at 180, eight
 // warps per SM left the shared loads' latency open, and a pass of training (four
-// epochs of these 16 samples with the copies) took 1558 us against 1500.
+// epochs of these 16 samples with the copies) took 1558 us against 1500.  Chained
+// launches (chain.cuh) of its fifteen kernels per minibatch take it to 1372.
 template <int CI, int CO, int OT, int RS>
 __global__ void __launch_bounds__(NTH, 2) conv_bwd_weight(const float* h, const float* dout, float* part, int N, int H, int Wd) {
+    lbk::chain_begin();
     constexpr int COP = (CO + 3) / 4 * 4, OG = COP / OT, PL = PLANE + 4, GP = COP == 32 ? COP + 4 : COP;
     static_assert(CI * OG * RS <= NTH && COP % OT == 0 && OT % 4 == 0 && NTH % COP == 0, "work split");
     extern __shared__ __align__(16) float sm[];
@@ -303,6 +306,7 @@ struct GradRows {
     int rows[NL];
 };
 __global__ void reduce_grads(const float* part, GradRows gr, int max_rows, int n, float* g) {
+    lbk::chain_begin();
     __shared__ float red[8][33];
     const int i = blockIdx.x * 32 + threadIdx.x % 32, share = threadIdx.x / 32;
     float s = 0.f;
@@ -374,6 +378,7 @@ __global__ void pack_weights(const float* p, __half* w16, int n) {
 
 __global__ void adam_pack(float* w, __half* w16, const float* g, float* m, float* v, int n, float lr, float b1, float b2,
                           float eps, float c1, float c2) {
+    lbk::chain_begin();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         store_packed(w16, i, adam_one(w, g, m, v, i, lr, b1, b2, eps, c1, c2));
 }
@@ -382,6 +387,7 @@ __global__ void adam_pack(float* w, __half* w16, const float* g, float* m, float
 // launch (two copies per sample and minibatch cost more than the kernels of the
 // thin layers).
 __global__ void gather_batch(const float* x, const float* t, const int* order, size_t nx, size_t nt, float* bx, float* bt) {
+    lbk::chain_begin();
     const float* sx = x + size_t(order[blockIdx.y]) * nx;
     const float* st = t + size_t(order[blockIdx.y]) * nt;
     float* dx = bx + size_t(blockIdx.y) * nx;
@@ -443,19 +449,19 @@ constexpr auto wgt_kernel = conv_bwd_weight<CI, CO, CO == 32 ? 8 : 4, CI == 32 &
 
 template <int CI, int CO, bool T>
 void launch_fwd(const lb_ws* w, int l, int n, int H, int Wd) {
-    fwd_kernel<CI, CO, T><<<conv_grid(n, H, Wd), NTH, smem_conv<CI, CO>(), w->st>>>(
-        w->act[l], w->p16 + PACK.ffwd[l], w->p + w->boff[l], nullptr, w->act[l + 1], H, Wd);
+    lbk::launch_chained(fwd_kernel<CI, CO, T>, conv_grid(n, H, Wd), NTH, smem_conv<CI, CO>(), w->st, w->act[l],
+                        w->p16 + PACK.ffwd[l], w->p + w->boff[l], nullptr, w->act[l + 1], H, Wd);
 }
 
 template <int CI, int CO>
 void launch_bwd(lb_ws* w, int l, int n, int H, int Wd) {
     const int ntiles = n * ((Wd + TILE - 1) / TILE) * ((H + TILE - 1) / TILE);
     w->rows.rows[l] = ntiles < 2 * w->sms ? ntiles : 2 * w->sms;
-    wgt_kernel<CI, CO><<<w->rows.rows[l], NTH, smem_bwd_w<CI, CO>(), w->st>>>(
-        w->act[l], w->dact[l + 1], w->part + size_t(2 * w->sms) * w->woff[l], n, H, Wd);
+    lbk::launch_chained(wgt_kernel<CI, CO>, w->rows.rows[l], NTH, smem_bwd_w<CI, CO>(), w->st, w->act[l], w->dact[l + 1],
+                        w->part + size_t(2 * w->sms) * w->woff[l], n, H, Wd);
     if constexpr (CI == LB_WS_HIDDEN)
-        bwd_kernel<CI, CO><<<conv_grid(n, H, Wd), NTH, smem_conv<CO, CI>(), w->st>>>(
-            w->dact[l + 1], w->p16 + PACK.fbwd[l], nullptr, w->act[l], w->dact[l], H, Wd);
+        lbk::launch_chained(bwd_kernel<CI, CO>, conv_grid(n, H, Wd), NTH, smem_conv<CO, CI>(), w->st, w->dact[l + 1],
+                            w->p16 + PACK.fbwd[l], nullptr, w->act[l], w->dact[l], H, Wd);
 }
 
 // Dynamic shared memory limits of the kernels, on the current device.
@@ -497,12 +503,12 @@ lb_status loss_grad(lb_ws* w, const float* t, int n, int H, int Wd, double* d_lo
     }
     forward(w, n, H, Wd);
     const size_t nout = size_t(n) * LB_WS_OUT * H * Wd;
-    mse_grad<<<256, 256, 0, w->st>>>(w->act[4], t, w->dact[4], nout, d_loss);
+    lbk::launch_chained(mse_grad, 256, 256, 0, w->st, w->act[4], t, w->dact[4], nout, d_loss);
     launch_bwd<LB_WS_HIDDEN, LB_WS_OUT>(w, 3, n, H, Wd);
     launch_bwd<LB_WS_HIDDEN, LB_WS_HIDDEN>(w, 2, n, H, Wd);
     launch_bwd<LB_WS_HIDDEN, LB_WS_HIDDEN>(w, 1, n, H, Wd);
     launch_bwd<LB_WS_IN, LB_WS_HIDDEN>(w, 0, n, H, Wd);
-    reduce_grads<<<(w->nparams + 31) / 32, 256, 0, w->st>>>(w->part, w->rows, 2 * w->sms, w->nparams, w->g);
+    lbk::launch_chained(reduce_grads, (w->nparams + 31) / 32, 256, 0, w->st, w->part, w->rows, 2 * w->sms, w->nparams, w->g);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(LB_ECUDA, std::string("warm-start backward: ") + cudaGetErrorString(e));
     return LB_OK;
@@ -690,12 +696,13 @@ lb_status lb_ws_train(lb_ws* w, const float* x, const float* t, int n, int H, in
             break;
         }
         for (int k = 0; k < nb && s == LB_OK; ++k) {
-            gather_batch<<<ggrid, 256, 0, w->st>>>(dx, dt, d_order + size_t(k) * batch, img * LB_WS_IN,
-                                                   img * LB_WS_OUT, w->act[0], bt);
+            lbk::launch_chained(gather_batch, ggrid, 256, 0, w->st, dx, dt, d_order + size_t(k) * batch, img * LB_WS_IN,
+                                img * LB_WS_OUT, w->act[0], bt);
             s = loss_grad(w, bt, batch, H, Wd, d_loss + k);
             ++w->adam_t;
             const float c1 = 1.f - std::pow(b1, float(w->adam_t)), c2 = 1.f - std::pow(b2, float(w->adam_t));
-            adam_pack<<<128, 256, 0, w->st>>>(w->p, w->p16, w->g, w->m, w->v, w->nparams, lr, b1, b2, eps, c1, c2);
+            lbk::launch_chained(adam_pack, 128, 256, 0, w->st, w->p, w->p16, w->g, w->m, w->v, w->nparams, lr, b1, b2, eps,
+                                c1, c2);
         }
         if (s != LB_OK) break;
         e = cudaMemcpyAsync(losses.data(), d_loss, size_t(nb) * sizeof(double), cudaMemcpyDeviceToHost, w->st);

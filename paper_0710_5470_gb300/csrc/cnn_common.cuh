@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "storage.cuh"   // lbk::widen
 
 namespace {
@@ -18,6 +19,7 @@ __device__ __forceinline__ int wrap(int v, int n) {
 // dy = 2 (y - t) / count; loss += sum (y - t)^2 / count (float64 accumulation;
 // launched with 256 threads).
 __global__ void mse_grad(const float* y, const float* t, float* dy, size_t n, double* loss) {
+    lbk::chain_begin();
     __shared__ double red[8];
     double acc = 0.0;
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
