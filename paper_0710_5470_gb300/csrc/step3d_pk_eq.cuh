@@ -133,7 +133,9 @@ struct PairCollEq {
     }
 };
 
-template <class S, int TX, int TY, int MINB, bool AOS>
+// HPF: the halo pairs' populations too are loaded a plane ahead; otherwise only the
+// own pair's, and the halo's at the head of their plane (38 registers less in float32).
+template <class S, int TX, int TY, int MINB, bool AOS, bool HPF = true>
 __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk_eq(const StepArgs args) {
     chain_begin();
     using L = D3Q19;
@@ -209,9 +211,10 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk_eq(const
     for (int m = 0; m < 1 + NAH; ++m) a_h[m] = AOS ? aos_bytes(a_in[m]) : 0u;
     float2 r0[1 + NAH];
     Wd ri[1 + NAH][18];
-    auto issue = [&]() {
+    auto issue = [&](int lo, int hi, int ld_off) {   // items lo .. hi - 1 of the plane at ld_off
 #pragma unroll
         for (int m = 0; m < 1 + NAH; ++m) {
+            if (m < lo || m >= hi) continue;
             if (m == 0 || a_rs[m] >= 0) {
                 const unsigned q = unsigned(ld_off) + a_in[m];
                 LB_GUARD(size_t(q) + 1 < nsites, BK_PK_LOAD, q, r0[m] = make_float2(0.f, 0.f);
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk_eq(const
             }
         }
     };
-    issue();
+    issue(0, HPF ? 1 + NAH : 1, ld_off);
 
     StencilAcc2 acc2{pp(0.f), pp(0.f), pp(0.f), pp(0.f), pp(0.f), pp(0.f), pp(0.f)};
     bool bad = false;
@@ -239,6 +242,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk_eq(const
         const int it = p - pstart;
         // ---------------- stage A: density of plane p; own pair into the stash
         {
+            if constexpr (!HPF) issue(1, 1 + NAH, ld_off);
             advance(ld_off);
             float* rho_w = rho_s + (it & 1) * Lay::RN;
             const int slot = it & 1;
@@ -273,7 +277,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_pk_eq(const
                     }
                 }
             }
-            if (p + 1 < pend) issue();
+            if (p + 1 < pend) issue(0, HPF ? 1 + NAH : 1, ld_off);
         }
         __syncthreads();
 
