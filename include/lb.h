@@ -112,7 +112,9 @@ lb_status lb_coexistence(double a, double b, double T, double* rho_l, double* rh
  * cuda_stream is a cudaStream_t (NULL = the legacy default stream); it must
  * outlive the context.  *out receives the context, or NULL on error.
  * D3Q19 float64 contexts also allocate a workspace of 11 (forcing scheme) or 1
- * float64 per site, at most 1 GiB; where it cannot be had they step without it.
+ * float64 per site, at most 1 GiB, and D3Q19 forcing contexts of 32-bit arithmetic
+ * whose step takes its densities from a field one float32 per site; where these
+ * cannot be had they step without them.
  * LB_EINVAL also for more than 2^31 - 1 sites (the kernels index sites with
  * 32-bit integers). */
 lb_status lb_create(const lb_params* p, void* cuda_stream, lb_ctx** out);
