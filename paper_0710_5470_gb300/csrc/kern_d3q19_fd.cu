@@ -8,17 +8,21 @@ using namespace lbk;
 
 namespace {
 
-template <class S, bool AOS, bool AL>
+cudaError_t density(const StepArgs& a, cudaStream_t st, void (*kernel)(const StepArgs, unsigned)) {
+    const unsigned pairs = (unsigned(a.nx) * unsigned(a.ny) * unsigned(a.nz) + 1u) / 2u;
+    return launch_chained(kernel, (pairs + 255u) / 256u, 256, 0, st, a, pairs);
+}
+
+template <class S, bool AOS>
 struct FDLaunch {
     static constexpr int TX = 32, TY = 8;
     using Lay = LayoutFD<TX, TY>;
     static_assert(Lay::BYTES <= 48 * 1024, "fits without opting in to more shared memory");
-    static const void* fn() { return reinterpret_cast<const void*>(step_kernel3d_fd<S, TX, TY, 3, AOS, AL>); }
+    static const void* fn() { return reinterpret_cast<const void*>(step_kernel3d_fd<S, TX, TY, 3, AOS>); }
     static cudaError_t step(const StepArgs& a, dim3 grid, cudaStream_t st) {
-        const unsigned pairs = (unsigned(a.nx) * unsigned(a.ny) * unsigned(a.nz) + 1u) / 2u;
-        const cudaError_t e = launch_chained(density_pairs<S, AOS>, (pairs + 255u) / 256u, 256, 0, st, a, pairs);
+        const cudaError_t e = density(a, st, density_pairs<S, AOS, PairIO<S>::RAW16>);
         return e != cudaSuccess ? e
-                                : launch_chained(step_kernel3d_fd<S, TX, TY, 3, AOS, AL>, grid, Lay::NTH, Lay::BYTES, st, a);
+                                : launch_chained(step_kernel3d_fd<S, TX, TY, 3, AOS>, grid, Lay::NTH, Lay::BYTES, st, a);
     }
     static LbKernelSet apply(LbKernelSet k, const char* name) {
         k.tx = TX;
@@ -34,12 +38,34 @@ struct FDLaunch {
     }
 };
 
+// Odd nx: one site per thread.
+template <class S>
+struct FD1Launch {
+    static constexpr int TX = 32, TY = 4, MINB = 4;
+    static const void* fn() { return reinterpret_cast<const void*>(step_kernel3d_fd1<S, TX, TY, MINB>); }
+    static cudaError_t step(const StepArgs& a, dim3 grid, cudaStream_t st) {
+        const cudaError_t e = density(a, st, density_pairs<S, false, false>);
+        return e != cudaSuccess ? e : launch_chained(step_kernel3d_fd1<S, TX, TY, MINB>, grid, TX * TY, 0, st, a);
+    }
+    static LbKernelSet apply(LbKernelSet k) {
+        k.tx = TX;
+        k.ty = TY;
+        k.threads = TX * TY;
+        k.smem = 0;
+        k.step_fn = fn();
+        k.step = &step;
+        k.step_pair_needs_even_nx = false;
+        k.name = "32x4, density field, one site per thread";
+        k.aos = false;
+        return k;
+    }
+};
+
 template <class S>
 LbKernelSet pick(int nx, LbKernelSet k) {
     if constexpr (PairIO<S>::RAW16)
-        if (nx % AOS_SITES == 0) return FDLaunch<S, true, true>::apply(k, "pairs 32x8, density field, interleaved blocks");
-    return nx % 2 == 0 ? FDLaunch<S, false, true>::apply(k, "pairs 32x8, density field")
-                       : FDLaunch<S, false, false>::apply(k, "pairs 32x8, density field, site by site");
+        if (nx % AOS_SITES == 0) return FDLaunch<S, true>::apply(k, "pairs 32x8, density field, interleaved blocks");
+    return nx % 2 == 0 ? FDLaunch<S, false>::apply(k, "pairs 32x8, density field") : FD1Launch<S>::apply(k);
 }
 
 }  // namespace
@@ -50,10 +76,12 @@ LbKernelSet pick(int nx, LbKernelSet k) {
 //     memory).  16^3 9.5 -> 8.7, 32^3 10.3 -> 9.6, 48^3 10.9 -> 10.4, 64^3 15.8 ->
 //     13.7, 96^3 42.9 -> 33.0, 128^3 92.2 -> 80.1, 256^3 728 -> 673, 320^3 1345 -> 1290,
 //     384^3 2342 -> 2397 (HBM);
-//   odd nx: the fused form is the one-site tile kernel.  fp16 deviations 9 x 10 x 11
-//     16.9 -> 13.3, 33 x 40 x 25 16.2 -> 13.9, 101 x 75 x 53 29.5 -> 23.7, 97 x 101 x 103
-//     62.2 -> 48.5, 201 x 190 x 180 347 -> 345, 221 x 220 x 210 443 -> 445; float32
-//     16.3 -> 12.7, 16.0 -> 12.0, 30.9 -> 23.4, 70.8 -> 52.9, 371 -> 381;
+//   odd nx: both forms take one site per thread; the fused one keeps a stash and two
+//     CTAs per SM.  fp16 deviations 9 x 10 x 11 16.8 -> 8.4, 33 x 40 x 25 15.8 -> 8.1, 101 x
+//     75 x 53 29.1 -> 20.6, 97 x 101 x 103 61.5 -> 44.7, 201 x 190 x 180 347 -> 262, 301 x 300 x
+//     300 1143 -> 907, 481 x 480 x 480 4832 -> 3612; float32 16.2 -> 8.6, 15.9 -> 8.4, 30.7 ->
+//     22.0, 70.6 -> 50.0, 370 -> 319, 1285 -> 1207, 5341 -> 5197: at every
+//     size, where the field can be had;
 //   16-bit, even nx, one array per population: 24^3 11.3 -> 9.1, 100 x 76 x 54
 //     23.9 -> 20.4, 200 x 190 x 180 251 -> 230;
 //   16-bit, interleaved blocks: 32^3 10.3 -> 9.4, 64^3 15.1 -> 13.2, 96^3 32.9 -> 28.6,
@@ -62,7 +90,7 @@ LbKernelSet pick(int nx, LbKernelSet k) {
 bool lbk_fd_wanted(int storage, int nx, size_t sites) {
     if (const char* e = std::getenv("LB_D3_FIELD")) return std::atoi(e) != 0;
     const double n = double(sites);
-    if (nx % 2 != 0) return n <= (storage == 1 ? 4e6 : 7e6);
+    if (nx % 2 != 0) return true;
     if (storage == 1) return n <= 4e7;
     return nx % AOS_SITES != 0 || n <= 3.4e6;
 }

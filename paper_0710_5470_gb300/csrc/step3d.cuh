@@ -154,6 +154,60 @@ __device__ __forceinline__ void start(StencilAcc<real>& a, const PlaneParts<real
     a.s = cur.s;
 }
 
+// Body force of one site (Eq. 28): the parts of plane q of M' added to the carries
+// -(U0(q-1) + U-(q-2)) and -U-(q-1); gf: the force of plane q - 1.  kc: the site's place
+// in the tile + 1 ring, rows of SX.
+template <class real>
+__device__ __forceinline__ void site_force_parts(const real* mpA, const real* mpB, int kc, int SX, real (&gacc1)[3],
+                                                 real (&gacc2)[3], real (&gf)[3]) {
+    real sp[3] = {0, 0, 0}, sz[3] = {0, 0, 0}, se[3] = {0, 0, 0};
+    real xx, xy, xz, yy, yz, zz;
+#pragma unroll
+    for (int sgn = -1; sgn <= 1; sgn += 2) {
+        const int kx = kc + sgn, ky = kc + sgn * SX;
+        const real s = real(sgn);
+        // x faces: s (Mxx, Mxy, Mxz); z parts (Mxz, Myz, Mzz)
+        ld4(mpA + 4 * kx, xx, xy, xz, yy);
+        ld2(mpB + 2 * kx, yz, zz);
+        sp[0] += s * xx; sp[1] += s * xy; sp[2] += s * xz;
+        sz[0] += xz; sz[1] += yz; sz[2] += zz;
+        // y faces: s (Mxy, Myy, Myz)
+        ld4(mpA + 4 * ky, xx, xy, xz, yy);
+        ld2(mpB + 2 * ky, yz, zz);
+        sp[0] += s * xy; sp[1] += s * yy; sp[2] += s * yz;
+        sz[0] += xz; sz[1] += yz; sz[2] += zz;
+        // xy diagonals (sx = sgn, sy = +-1)
+#pragma unroll
+        for (int sgy = -1; sgy <= 1; sgy += 2) {
+            const int ke = kc + sgn + sgy * SX;
+            const real ty_ = real(sgy);
+            ld4(mpA + 4 * ke, xx, xy, xz, yy);
+            ld2(mpB + 2 * ke, yz, zz);
+            se[0] += s * xx + ty_ * xy;
+            se[1] += s * xy + ty_ * yy;
+            se[2] += s * xz + ty_ * yz;
+        }
+    }
+    ld4(mpA + 4 * kc, xx, xy, xz, yy);
+    ld2(mpB + 2 * kc, yz, zz);
+    const real zc[3] = {xz, yz, zz};
+    const real sixth = real(1) / real(6), twelfth = real(1) / real(12);
+    real up[3], u0[3], um[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        u0[c] = sixth * sp[c] + twelfth * se[c];
+        up[c] = twelfth * (sp[c] + sz[c]) + sixth * zc[c];
+        um[c] = twelfth * (sp[c] - sz[c]) - sixth * zc[c];
+    }
+    // g(q-1) = -(U+(q) + U0(q-1) + U-(q-2))   (Eq. 28)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        gf[c] = gacc1[c] - up[c];
+        gacc1[c] = gacc2[c] - u0[c];
+        gacc2[c] = -um[c];
+    }
+}
+
 // PAIR: stage A moves two adjacent x sites per thread with 2-vector loads
 // (requires an even nx); otherwise one site per thread.
 template <bool FORCING, class S, int TX, int TY, bool PAIR>
@@ -380,53 +434,7 @@ __global__ void __launch_bounds__(TX* TY, (sizeof(typename S::real) == 4 && TX *
         real gf[3] = {0, 0, 0};
         if constexpr (FORCING) {
             if (assemble_q) {
-                const int kc = (ty + 1) * SX + (tx + 1);
-                real sp[3] = {0, 0, 0}, sz[3] = {0, 0, 0}, se[3] = {0, 0, 0};
-                real xx, xy, xz, yy, yz, zz;
-#pragma unroll
-                for (int sgn = -1; sgn <= 1; sgn += 2) {
-                    const int kx = kc + sgn, ky = kc + sgn * SX;
-                    const real s = real(sgn);
-                    // x faces: s (Mxx, Mxy, Mxz); z parts (Mxz, Myz, Mzz)
-                    ld4(mpA + 4 * kx, xx, xy, xz, yy);
-                    ld2(mpB + 2 * kx, yz, zz);
-                    sp[0] += s * xx; sp[1] += s * xy; sp[2] += s * xz;
-                    sz[0] += xz; sz[1] += yz; sz[2] += zz;
-                    // y faces: s (Mxy, Myy, Myz)
-                    ld4(mpA + 4 * ky, xx, xy, xz, yy);
-                    ld2(mpB + 2 * ky, yz, zz);
-                    sp[0] += s * xy; sp[1] += s * yy; sp[2] += s * yz;
-                    sz[0] += xz; sz[1] += yz; sz[2] += zz;
-                    // xy diagonals (sx = sgn, sy = +-1)
-#pragma unroll
-                    for (int sgy = -1; sgy <= 1; sgy += 2) {
-                        const int ke = kc + sgn + sgy * SX;
-                        const real ty_ = real(sgy);
-                        ld4(mpA + 4 * ke, xx, xy, xz, yy);
-                        ld2(mpB + 2 * ke, yz, zz);
-                        se[0] += s * xx + ty_ * xy;
-                        se[1] += s * xy + ty_ * yy;
-                        se[2] += s * xz + ty_ * yz;
-                    }
-                }
-                ld4(mpA + 4 * kc, xx, xy, xz, yy);
-                ld2(mpB + 2 * kc, yz, zz);
-                const real zc[3] = {xz, yz, zz};
-                const real sixth = real(1) / real(6), twelfth = real(1) / real(12);
-                real up[3], u0[3], um[3];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    u0[c] = sixth * sp[c] + twelfth * se[c];
-                    up[c] = twelfth * (sp[c] + sz[c]) + sixth * zc[c];
-                    um[c] = twelfth * (sp[c] - sz[c]) - sixth * zc[c];
-                }
-                // g(q-1) = -(U+(q) + U0(q-1) + U-(q-2))   (Eq. 28)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    gf[c] = gacc1[c] - up[c];
-                    gacc1[c] = gacc2[c] - u0[c];
-                    gacc2[c] = -um[c];
-                }
+                site_force_parts(mpA, mpB, (ty + 1) * SX + (tx + 1), SX, gacc1, gacc2, gf);
             }
         }
 

@@ -14,26 +14,24 @@
 // either storage, 472 instructions per site where the fused form has 576 (fp16
 // deviations).  Both are bound by latency and by the shared-memory pipe (M' of
 // twelve sites per pair and plane), so the lighter kernel gains where the fused one
-// has fewer CTAs (float32), where the fused one takes one site per thread (odd nx)
-// and where the second pass reads from L2; kern_d3q19_fd.cu has the measurements
+// has fewer CTAs (float32) and where the second pass reads from L2; kern_d3q19_fd.cu has the measurements
 // and the lines.  Carries in thread-private shared memory allow four or five CTAs
 // per SM but took 75 instead of 67 us (128^3, fp16 deviations).  The density sums
 // keep their order: both forms give the same bits.
 //
-// AL: nx even, so that pairs are aligned 2-vectors and never split by the
-// periodic wrap; otherwise (odd nx) every site of a pair is loaded and stored on
-// its own, wrapped on its own, and a pair whose second site lies beyond the
-// lattice stores its first site only.
+// Odd nx: one site per thread (step_kernel3d_fd1), since pairs would be split by the
+// periodic wrap and by every second row's alignment.
 #pragma once
 #include "chain.cuh"
-#include "step2d_pk.cuh"   // ld_split
+#include "step3d.cuh"
 #include "step3d_pk.cuh"
 
 namespace lbk {
 
 // Density of two sites adjacent in memory per thread: the lattice as a row of
-// sites, whatever its shape (the arrays are padded to whole 128-site rows).
-template <class S, bool AOS>
+// sites, whatever its shape (the arrays are padded to whole 128-site rows).  MIXED:
+// the sums of the step that follows (pair_rho).
+template <class S, bool AOS, bool MIXED>
 __global__ void __launch_bounds__(256) density_pairs(const StepArgs a, unsigned pairs) {
     chain_begin();
     using IO = PairIO<S>;
@@ -52,7 +50,7 @@ __global__ void __launch_bounds__(256) density_pairs(const StepArgs a, unsigned 
             w[i - 1] = IO::ld(a.src[i], q);
         });
     }
-    reinterpret_cast<float2*>(a.rho32)[t] = pair_rho<S, IO::RAW16>(f0, w, a.rsum).v;
+    reinterpret_cast<float2*>(a.rho32)[t] = pair_rho<S, MIXED>(f0, w, a.rsum).v;
 }
 
 template <int TX, int TY>
@@ -64,7 +62,7 @@ struct LayoutFD {
     static constexpr size_t BYTES = OFF_MPB + size_t(SN) * 8;
 };
 
-template <class S, int TX, int TY, int MINB, bool AOS, bool AL>
+template <class S, int TX, int TY, int MINB, bool AOS>
 __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const StepArgs args) {
     chain_begin();
     using L = D3Q19;
@@ -75,7 +73,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
     constexpr bool RAW16 = IO::RAW16;
     constexpr int H = Lay::H, HX = Lay::HX, TXP = Lay::TXP, NTH = Lay::NTH;
     constexpr int RX = Lay::RX, SX = Lay::SX, NBR = Lay::NBR;
-    static_assert(!AOS || (RAW16 && AL), "interleaved layout: 16-bit storage, nx a multiple of 32");
+    static_assert(!AOS || RAW16, "interleaved layout: 16-bit storage, nx a multiple of 32");
     constexpr int ROWB = 2 * AOS_SITES;             // bytes of one population row of a block
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -96,17 +94,16 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
     const float pk = args.fkappa;
     const float* field = args.rho32;
 
-    // ---- region items of the density: pairs (AL) or single sites, in-plane
-    // element index and place in the slot
-    constexpr int W = AL ? 2 : 1, NIT = Lay::RN / W, NA = (NIT + NTH - 1) / NTH, RXW = RX / W;
+    // ---- region pairs of the density: in-plane element index and place in the slot
+    constexpr int NIT = Lay::NIT, NA = (NIT + NTH - 1) / NTH, RXP = Lay::RXP;
     unsigned a_in[NA];
 #pragma unroll
     for (int m = 0; m < NA; ++m) {
         const int k = tid + m * NTH;
-        a_in[m] = k < NIT ? unsigned(wrapi(y0 - H + k / RXW, ny) * nx + wrapi(x0 - HX + (k % RXW) * W, nx)) : 0u;
+        a_in[m] = k < NIT ? unsigned(wrapi(y0 - H + k / RXP, ny) * nx + wrapi(x0 - HX + (k % RXP) * 2, nx)) : 0u;
     }
     const int xo = x0 + 2 * px, yo = y0 + py;
-    const bool own = xo < nx && yo < ny, own1 = own && (AL || xo + 1 < nx);
+    const bool own = xo < nx && yo < ny;
     // ---- ring items of stage B: region index and M' index
     int b_rc[NBR], b_mp[NBR];
 #pragma unroll
@@ -128,10 +125,10 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
     const int mp0 = Lay::mp_index(2 * px + 1, py + 1), mp1 = Lay::mp_index(2 * px + 2, py + 1);
     // push targets: x columns of the pair's neighbours, row offsets of the pair
     const unsigned xm1 = unsigned(wrapi(xo - 1, nx)), xc = unsigned(wrapi(xo, nx));
-    const unsigned xp1 = AL ? xc + 1 : unsigned(wrapi(xo + 1, nx)), xp2 = unsigned(wrapi(xo + 2, nx));
+    const unsigned xp1 = xc + 1, xp2 = unsigned(wrapi(xo + 2, nx));
     const unsigned yr[3] = {unsigned(wrapi(yo - 1, ny) * nx), unsigned(wrapi(yo, ny) * nx),
                             unsigned(wrapi(yo + 1, ny) * nx)};
-    const unsigned q_in = yr[1] + xc, q_in1 = yr[1] + xp1;
+    const unsigned q_in = yr[1] + xc;
 
     const int pstart = z0 - 2, pend = z1 + 2;
     const int vol = nz * plane;
@@ -148,9 +145,8 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
         for (int m = 0; m < NA; ++m) {
             if (tid + m * NTH < NIT) {
                 const unsigned q = unsigned(ld_off) + a_in[m];
-                LB_GUARD(size_t(q) + W - 1 < nsites, BK_PK_LOAD, q, rn[m] = make_float2(0.f, 0.f); continue)
-                if constexpr (AL) rn[m] = reinterpret_cast<const float2*>(field)[q >> 1];
-                else rn[m].x = field[q];
+                LB_GUARD(size_t(q) + 1 < nsites, BK_PK_LOAD, q, rn[m] = make_float2(0.f, 0.f); continue)
+                rn[m] = reinterpret_cast<const float2*>(field)[q >> 1];
             }
         }
         advance(ld_off);
@@ -176,23 +172,18 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
 #pragma unroll
         for (int m = 0; m < NA; ++m) {
             const int k = tid + m * NTH;
-            if (k < NIT) {
-                if constexpr (AL) *reinterpret_cast<float2*>(rho_p + 2 * k) = rn[m];
-                else rho_p[k] = rn[m].x;
-            }
+            if (k < NIT) *reinterpret_cast<float2*>(rho_p + 2 * k) = rn[m];
         }
         if (p + 1 < pend) issue();
         float2 f0 = make_float2(0.f, 0.f);
         Wd w[18];
         if (s >= z0) {
-            const unsigned q = unsigned(zr[1]) + q_in, q1 = unsigned(zr[1]) + q_in1;
+            const unsigned q = unsigned(zr[1]) + q_in;
 #ifdef LB_DEBUG_BOUNDS
-            if (lbk::in_bounds(size_t(q) < nsites && size_t(q1) < nsites, BK_PK_LOAD, q))
+            if (lbk::in_bounds(size_t(q) + 1 < nsites, BK_PK_LOAD, q))
 #endif
             {
-                if constexpr (AL) f0 = reinterpret_cast<const float2*>(args.src_base)[q >> 1];
-                else f0 = make_float2(reinterpret_cast<const float*>(args.src_base)[q],
-                                      reinterpret_cast<const float*>(args.src_base)[q1]);
+                f0 = reinterpret_cast<const float2*>(args.src_base)[q >> 1];
                 if constexpr (AOS) {
                     const char* b = args.src[1] + size_t(q / AOS_SITES) * (2 * AOS_BLOCK_HALVES) + (q % AOS_SITES) * 2;
 #pragma unroll
@@ -200,8 +191,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
                 } else {
                     static_for<1, 19>([&](auto I) {
                         constexpr int i = decltype(I)::value;
-                        if constexpr (AL) w[i - 1] = IO::ld(args.src[i], q);
-                        else w[i - 1] = ld_split<S>(args.src[i], q, q1);
+                        w[i - 1] = IO::ld(args.src[i], q);
                     });
                 }
             }
@@ -257,7 +247,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
         if (s >= z0) {
             const P2 rho = c2;
             const P2 G[3] = {Gc[0], Gc[1], Gc[2]};
-            bad |= (own && (!(rho.v.x > 0.f) || !(rho.v.x < 1e30f))) || (own1 && (!(rho.v.y > 0.f) || !(rho.v.y < 1e30f)));
+            bad |= own && (!(rho.v.x > 0.f) || !(rho.v.x < 1e30f) || !(rho.v.y > 0.f) || !(rho.v.y < 1e30f));
             P2 j[3];
             if constexpr (RAW16) pair_momentum_mixed<S>(w, j);
             else pair_momentum<S>(w, j);
@@ -297,26 +287,19 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
                             IO::st1p(b + cb[0], v.v.x);
                             IO::st1p(b + cb[1], v.v.y);
                         }
-                    } else if constexpr (AL && ex == 0) {
+                    } else if constexpr (ex == 0) {
                         IO::st2(args.dst[i], row + xc, v);
                     } else {
                         IO::st1(args.dst[i], row + xa, v.v.x);
-                        if (own1) IO::st1(args.dst[i], row + xb, v.v.y);
+                        IO::st1(args.dst[i], row + xb, v.v.y);
                     }
                 };
                 const P2 o0 = fma(K.omw, P2{f0}, K.c0);
                 const unsigned q = unsigned(zr[1]) + q_in;
 #ifdef LB_DEBUG_BOUNDS
-                if (lbk::in_bounds(size_t(q) < nsites && size_t(unsigned(zr[1])) + q_in1 < nsites, BK_PK_STORE, q))
+                if (lbk::in_bounds(size_t(q) + 1 < nsites, BK_PK_STORE, q))
 #endif
-                {
-                    if constexpr (AL) {
-                        reinterpret_cast<float2*>(args.dst_base)[q >> 1] = o0.v;
-                    } else {
-                        reinterpret_cast<float*>(args.dst_base)[q] = o0.v.x;
-                        if (own1) reinterpret_cast<float*>(args.dst_base)[unsigned(zr[1]) + q_in1] = o0.v.y;
-                    }
-                }
+                    reinterpret_cast<float2*>(args.dst_base)[q >> 1] = o0.v;
                 static_for<1, 19>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     constexpr int o = opposite<L>(i);
@@ -326,6 +309,180 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
                         store(std::integral_constant<int, i>{}, oi);
                         store(std::integral_constant<int, o>{}, on);
                     }
+                });
+            }
+            advance(zr[0]);
+            advance(zr[1]);
+            advance(zr[2]);
+        }
+        if (assemble) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) Gc[c] = Gn[c];
+            lapc = lapn;
+        }
+        c2 = c1;
+        c1 = cn;
+    }
+    if (bad) atomicOr(args.status, 1u);
+}
+
+// The same step for an odd nx, one site per thread: the arithmetic of step_kernel3d
+// (step3d.cuh) function by function, the density pass in its order too, so that both
+// forms give the same bits; a last-bit difference would flip roundings to 16 bits.  A
+// thread carries its own site's gradient and density in registers and takes at most one of
+// the ring's sites; no stash, 6 KB of shared memory, four CTAs of 32 x 4 sites per SM (126
+// registers).  Measured on a GB300, us per step at 101 x 75 x 53, bf16 deviations: one-site
+// fused kernel 29.1, this 20.8, 32 x 8 tiles with two CTAs per SM 22.6, 32 x 4 with five
+// 22.7, pairs split site by site 22.7.
+template <class S, int TX, int TY, int MINB>
+__global__ void __launch_bounds__(TX* TY, MINB) step_kernel3d_fd1(const StepArgs args) {
+    chain_begin();
+    using L = D3Q19;
+    constexpr int Q = 19, H = 2, NT = TX * TY;
+    constexpr int RX = TX + 2 * H, RY = TY + 2 * H, RN = RX * RY;
+    constexpr int SX = TX + 2, SY = TY + 2, SN = SX * SY, NRING = SN - NT;
+    constexpr int NA = (RN + NT - 1) / NT;
+    static_assert(NRING <= NT, "one ring site per thread");
+    __shared__ float rho_s[2 * RN];
+    __shared__ __align__(16) float mpA[4 * SN];   // (Mxx, Mxy, Mxz, Myy) per ring-1 site
+    __shared__ __align__(8) float mpB[2 * SN];    // (Myz, Mzz) per ring-1 site
+
+    const int nx = args.nx, ny = args.ny, nz = args.nz;
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    const int4 wk = args.work[blockIdx.x];
+    const int x0 = wk.x, y0 = wk.y, z0 = wk.z, z1 = wk.w;
+    const int plane = nx * ny, vol = nz * plane;
+    const float pk = args.fkappa;
+
+    int a_in[NA];
+#pragma unroll
+    for (int m = 0; m < NA; ++m) {
+        const int k = tid + m * NT;
+        a_in[m] = k < RN ? wrapi(y0 - H + k / RX, ny) * nx + wrapi(x0 - H + k % RX, nx) : 0;
+    }
+    // stage-B sites: the own one and, for the first NRING threads, one of the ring
+    const int rc = (ty + H) * RX + tx + H, kc = (ty + 1) * SX + tx + 1;
+    int b_rc = -1, b_k = 0;
+    if (tid < NRING) {
+        int sx, sy;
+        if (tid < 2 * SX) {
+            sx = tid % SX;
+            sy = tid < SX ? 0 : SY - 1;
+        } else {
+            const int k = tid - 2 * SX;
+            sy = 1 + (k >> 1);
+            sx = (k & 1) ? SX - 1 : 0;
+        }
+        b_rc = (sy + H - 1) * RX + (sx + H - 1);
+        b_k = sy * SX + sx;
+    }
+    const int xs = x0 + tx, ys = y0 + ty;
+    const bool own = xs < nx && ys < ny;
+    const int xw[3] = {wrapi(xs - 1, nx), wrapi(xs, nx), wrapi(xs + 1, nx)};
+    const int yr[3] = {wrapi(ys - 1, ny) * nx, wrapi(ys, ny) * nx, wrapi(ys + 1, ny) * nx};
+
+    const int pstart = z0 - 2, pend = z1 + 2;
+    int ld_off = wrapi(pstart, nz) * plane;
+    int zr[3] = {wrapi(z0 - 1, nz) * plane, wrapi(z0, nz) * plane, wrapi(z0 + 1, nz) * plane};
+    auto advance = [&](int& v) {
+        v += plane;
+        if (v == vol) v = 0;
+    };
+    float rn[NA];
+    auto issue = [&]() {   // density of plane ld_off on the region
+#pragma unroll
+        for (int m = 0; m < NA; ++m) {
+            if (tid + m * NT < RN) {
+                const unsigned q = unsigned(ld_off + a_in[m]);
+                LB_GUARD(q < unsigned(vol), BK_3D_LOAD, q, rn[m] = 0.f; continue)
+                rn[m] = args.rho32[q];
+            }
+        }
+        advance(ld_off);
+    };
+    issue();
+
+    StencilAcc<float> acc{0, 0, 0, 0, 0, 0, 0}, accr{0, 0, 0, 0, 0, 0, 0};   // own site, ring site
+    float gacc1[3] = {0, 0, 0}, gacc2[3] = {0, 0, 0};
+    float Gc[3] = {0, 0, 0}, lapc = 0, c1 = 0, c2 = 0;   // G, lap one plane back, rho one and two
+    bool bad = false;
+
+    for (int p = pstart; p < pend; ++p) {
+        const int it = p - pstart, s = p - 2;
+        float* rho_p = rho_s + (it & 1) * RN;
+#pragma unroll
+        for (int m = 0; m < NA; ++m)
+            if (tid + m * NT < RN) rho_p[tid + m * NT] = rn[m];
+        if (p + 1 < pend) issue();
+        typename S::raw0 r0{};
+        typename S::rawi ri[Q - 1];
+        if (s >= z0) {   // populations of the site collided at the end of this turn
+            const unsigned q = unsigned(zr[1] + yr[1] + xw[1]);
+#ifdef LB_DEBUG_BOUNDS
+            if (lbk::in_bounds(q < unsigned(vol), BK_3D_LOAD, q))
+#endif
+            {
+                r0 = S::ld0(args.src[0], q);
+                static_for<1, Q>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    ri[i - 1] = S::ldi(args.src[i], q);
+                });
+            }
+        }
+        __syncthreads();
+
+        // ---------------- stage B: stencil parts of plane p; G, lap and M' of plane p - 1
+        const bool assemble = it >= 2;
+        float Gn[3] = {0, 0, 0}, lapn = 0, cn;
+        {
+            auto put = [&](int k, const float (&G)[3]) {
+                const float g2 = G[0] * G[0] + G[1] * G[1] + G[2] * G[2];
+                const float hk = 0.5f * pk * g2;
+                LB_GUARD(k >= 0 && k < SN, BK_PK_SHARED, k, return)
+                st4(mpA + 4 * k, pk * G[0] * G[0] - hk, pk * G[0] * G[1], pk * G[0] * G[2], pk * G[1] * G[1] - hk);
+                st_pair(mpB + 2 * k, pk * G[1] * G[2], pk * G[2] * G[2] - hk);
+            };
+            const PlaneParts<float> cur = plane_parts(rho_p, rc, RX);
+            cn = cur.c;
+            if (assemble) {
+                finish(acc, cur, Gn, lapn);
+                put(kc, Gn);
+            }
+            start(acc, cur);
+            if (b_rc >= 0) {
+                const PlaneParts<float> cr = plane_parts(rho_p, b_rc, RX);
+                if (assemble) {
+                    float G[3], lap;
+                    finish(accr, cr, G, lap);
+                    put(b_k, G);
+                }
+                start(accr, cr);
+            }
+        }
+        __syncthreads();
+
+        // ---------------- body force: parts of plane p - 1 (Eq. 28)
+        float gf[3] = {0, 0, 0};
+        if (assemble) site_force_parts(mpA, mpB, kc, SX, gacc1, gacc2, gf);
+
+        // ---------------- stage C: collide and push plane s = p - 2
+        if (s >= z0) {
+            if (own) {
+                float f[Q], out[Q];
+                f[0] = S::dec0(r0);
+                static_for<1, Q>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    f[i] = S::devi(ri[i - 1]);
+                });
+                bad |= !(c2 > 0.f) || !(c2 < 1e30f);
+                collide<L, true, float>(f, c2, Gc, lapc, gf, args.fa, args.fb, args.fT, pk, args.fomega, args.fnu,
+                                        args.pref, args.rsum, out);
+                static_for<0, Q>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    const int idx = zr[1 + L::ez(i)] + yr[1 + L::ey(i)] + xw[1 + L::ex(i)];
+                    LB_GUARD(idx >= 0 && idx < vol, BK_3D_STORE, idx, return)
+                    if constexpr (i == 0) S::st0(args.dst[0], size_t(idx), out[0]);
+                    else S::sti(args.dst[i], size_t(idx), out[i]);
                 });
             }
             advance(zr[0]);
