@@ -6,7 +6,7 @@
 // multiplication and FMA counts alike, while loads, shared memory and integer
 // work are free beside them.  Hence
 //   * the stencils, the body force and the collision are written for the fewest
-//     operations (136 per site and step in the forcing scheme where the
+//     operations (138 per site and step in the forcing scheme where the
 //     lattice-generic form took about 230): common differences are shared, the
 //     factors 1/12 and 1/6 of the stencils go into constants of the host, M'
 //     has two components (M'_xx = -M'_yy), one division gives both reciprocals;
@@ -15,9 +15,9 @@
 //     TX * TY) first, which sit on other schedulers;
 //   * the tile is chosen by the lattice's size (kern_d2q9.cu).
 // Measured on a GB300 (us per step, forcing / equilibrium scheme, the
-// lattice-generic kernel on 32 x 8 tiles -> now): 100^2 18.7 -> 7.5 / 14.2 -> 6.4,
-// 256^2 33.8 -> 23.4 / 25.1 -> 18.7, 512^2 114 -> 76 / 83 -> 62, 1024^2 434 -> 289 /
-// 315 -> 236 (3.6 G sites/s; with 155 operations per site, halo included, 90% of
+// lattice-generic kernel on 32 x 8 tiles -> now, launches chained): 100^2 18.2 -> 6.9 /
+// 13.6 -> 5.8, 200^2 33.4 -> 17.2 / 24.6 -> 13.1, 512^2 113 -> 76 / 82 -> 63, 1024^2 432 ->
+// 292 / 313 -> 239 (3.6 G sites/s; with 157 operations per site, halo included, 90% of
 // the FP64 pipe).
 #pragma once
 #include "chain.cuh"
@@ -81,7 +81,9 @@ __device__ __forceinline__ void collide9_f64(const double (&f)[9], double rho, d
     const double jx = a1 + (a5 - a7), jy = a3 + (a5 + a7);
     const double ob = fma(-k.b, rho, 1.0);
     const double r = 1.0 / (rho * ob);
-    const double irho = r * ob, ib = r * rho;
+    const double irho = r * ob, ib0 = r * rho;
+    // 1 / (1 - b rho) to half a unit (one Newton step): p0 multiplies its error several times (collide19_f64)
+    const double ib = fma(ib0, fma(-ob, ib0, 1.0), ib0);
     const double ux = jx * irho, uy = jy * irho;
     const double Tib = k.T * ib;
     const double p0 = rho * fma(-k.a, rho, Tib);                                      // Eq. 2

@@ -1,7 +1,7 @@
 // D3Q19 time step in float64: two or three passes over one-site threads.
 //
 // What bounds float64 on a GB300 is the FP64 pipe (two lanes per clock and SM):
-// at 299 operations per site the forcing step needs 0.48 ns of the whole chip
+// at 301 operations per site the forcing step needs 0.48 ns of the whole chip
 // per site, while its 600 bytes of traffic need 0.09 ns.  So the step is cut
 // where that removes operations, and moves the intermediate fields through
 // memory (mostly L2) instead of recomputing them:
@@ -9,13 +9,13 @@
 //   mprime3_f64    (forcing) G' = 12 grad rho, lap' = 6 lap rho (Eq. 29) and
 //                  M'_ab - delta_ab M'_cc / 2 over 12: 52;
 //   collide3_f64   the force -div M' (Eq. 28), the collision (Eqs. 2-6, 27, 36)
-//                  and the push (Eq. 4): 229; (equilibrium) its own G', lap'.
+//                  and the push (Eq. 4): 231; (equilibrium) its own G', lap'.
 // The fused kernel of step3d.cuh, which marches 32 x 4 tiles through z,
 // recomputed the densities of 2.25 and the M' of 1.6 sites per site and spent
 // about 520 operations, in one long chain per CTA.  Measured, us per step, fused
-// -> passes, forcing and equilibrium scheme: 32^3 97 -> 26 and 52 -> 19, 64^3 264
-// -> 162 and 165 -> 120, 128^3 1887 -> 1194 and 1308 -> 896 (1.76 and 2.34 G
-// sites/s, the FP64 pipe 85% busy).
+// -> passes, forcing and equilibrium scheme (launches chained): 32^3 96 -> 23.6 and 51 ->
+// 17.5, 64^3 263 -> 159 and 164 -> 119, 128^3 1884 -> 1198 and 1305 -> 898 (1.75 and 2.34
+// G sites/s, the FP64 pipe 85% busy).
 //
 // The fields live in a workspace of the context: the whole lattice where that
 // fits its limit, else slabs of planes with two (forcing) or one halo planes on
@@ -211,7 +211,7 @@ __device__ __forceinline__ void body_force19_f64(const double* M, long long fiel
 // collide() of step_kernel.cuh for D3Q19 float64 from G', lap' and the force g:
 // the same quadratic form in e_i, with S_ab = omega Q_ab + u_a g_b + u_b g_a; the
 // even part of an axis pair is E_c = Aw/6 + S_cc/4, that of a diagonal pair
-// (E_c + E_d)/2 - Aw/12 +- S_cd/4.  150 operations.
+// Aw/12 + (S_cc + S_dd)/8 +- S_cd/4.  152 operations.
 template <bool FORCING, class Push>
 __device__ __forceinline__ void collide19_f64(const double (&f)[19], double rho, const double (&G)[3], double lap,
                                               const double (&g)[3], const Consts64x3& k, Push&& push) {
@@ -226,7 +226,11 @@ __device__ __forceinline__ void collide19_f64(const double (&f)[19], double rho,
     }
     const double ob = fma(-k.b, rho, 1.0);
     const double r = 1.0 / (rho * ob);
-    const double irho = r * ob, ib = r * rho;
+    const double irho = r * ob, ib0 = r * rho;
+    // 1 / (1 - b rho) to half a unit: p0 is a small difference of T ib and a rho, which multiplies the error
+    // of ib several times (one Newton step, two operations; without it the populations' error against
+    // exact arithmetic was 7 - 17% larger, 20 steps of a drop)
+    const double ib = fma(ib0, fma(-ob, ib0, 1.0), ib0);
     const double Tib = k.T * ib;
     const double p0 = rho * fma(-k.a, rho, Tib);                                     // Eq. 2
     const double olam = fma(-k.onu12x3, Tib * ib, fma(k.onu12x6a, rho, k.onu12));    // omega lambda/12, Eq. 36
@@ -252,14 +256,14 @@ __device__ __forceinline__ void collide19_f64(const double (&f)[19], double rho,
     double Aw = fma(-0.5, fma(oj[0], u[0], fma(oj[1], u[1], oj[2] * u[2])), k.omega * fma(-(k.kap6 * rho), lap, p0));
     Aw = fma(-2.5, ohh, Aw);
     if constexpr (FORCING) Aw -= fma(u[0], g[0], fma(u[1], g[1], u[2] * g[2]));
-    const double A6 = Aw * (1.0 / 6.0), hA = -0.5 * A6;
+    const double A6 = Aw * (1.0 / 6.0), hA = 0.5 * A6;
     double E[3], P[3][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) E[c] = fma(0.25, S[c][c], A6);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int d = c + 1; d < 3; ++d) P[c][d] = fma(0.5, E[c] + E[d], hA);
+        for (int d = c + 1; d < 3; ++d) P[c][d] = fma(0.125, S[c][c] + S[d][d], hA);
     if constexpr (!FORCING) {
         // omega w^ab kappa d_a rho d_b rho: on an axis 5/12 of its own diagonal term and -1/3 of
         // the others; on a diagonal -1/24 of the two it touches, 1/12 of the third and +-1/4 of M_cd
