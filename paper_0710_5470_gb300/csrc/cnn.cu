@@ -699,6 +699,7 @@ lb_status lb_ws_train(lb_ws* w, const float* x, const float* t, int n, int H, in
             lbk::launch_chained(gather_batch, ggrid, 256, 0, w->st, dx, dt, d_order + size_t(k) * batch, img * LB_WS_IN,
                                 img * LB_WS_OUT, w->act[0], bt);
             s = loss_grad(w, bt, batch, H, Wd, d_loss + k);
+            if (s != LB_OK) break;   // no optimiser step without a gradient
             ++w->adam_t;
             const float c1 = 1.f - std::pow(b1, float(w->adam_t)), c2 = 1.f - std::pow(b2, float(w->adam_t));
             lbk::launch_chained(adam_pack, 128, 256, 0, w->st, w->p, w->p16, w->g, w->m, w->v, w->nparams, lr, b1, b2, eps,
