@@ -494,6 +494,12 @@ cudaError_t forward(lb_ws* w, int n, int H, int Wd) {
     return cudaGetLastError();
 }
 
+// A launch of the training loop that was refused; the error is reported, not left for the next call.
+lb_status launch_failed(cudaError_t e) {
+    cudaGetLastError();
+    return fail(LB_ECUDA, std::string("training launch: ") + cudaGetErrorString(e));
+}
+
 // loss (added to *d_loss, zeroed by the caller) and gradients of the batch whose inputs sit in act[0], targets in t
 lb_status loss_grad(lb_ws* w, const float* t, int n, int H, int Wd, double* d_loss) {
     if (!w->part && cudaMalloc(&w->part, size_t(2 * w->sms) * w->nparams * sizeof(float)) != cudaSuccess) {
@@ -501,7 +507,9 @@ lb_status loss_grad(lb_ws* w, const float* t, int n, int H, int Wd, double* d_lo
         w->part = nullptr;
         return fail(LB_ENOMEM, "partial gradients");
     }
-    forward(w, n, H, Wd);
+    cudaGetLastError();   // an error that an earlier call of the program left is not this one's
+    cudaError_t e = forward(w, n, H, Wd);
+    if (e != cudaSuccess) return fail(LB_ECUDA, std::string("warm-start forward launch: ") + cudaGetErrorString(e));
     const size_t nout = size_t(n) * LB_WS_OUT * H * Wd;
     lbk::launch_chained(mse_grad, 256, 256, 0, w->st, w->act[4], t, w->dact[4], nout, d_loss);
     launch_bwd<LB_WS_HIDDEN, LB_WS_OUT>(w, 3, n, H, Wd);
@@ -509,7 +517,7 @@ lb_status loss_grad(lb_ws* w, const float* t, int n, int H, int Wd, double* d_lo
     launch_bwd<LB_WS_HIDDEN, LB_WS_HIDDEN>(w, 1, n, H, Wd);
     launch_bwd<LB_WS_IN, LB_WS_HIDDEN>(w, 0, n, H, Wd);
     lbk::launch_chained(reduce_grads, (w->nparams + 31) / 32, 256, 0, w->st, w->part, w->rows, 2 * w->sms, w->nparams, w->g);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return fail(LB_ECUDA, std::string("warm-start backward: ") + cudaGetErrorString(e));
     return LB_OK;
 }
@@ -696,14 +704,15 @@ lb_status lb_ws_train(lb_ws* w, const float* x, const float* t, int n, int H, in
             break;
         }
         for (int k = 0; k < nb && s == LB_OK; ++k) {
-            lbk::launch_chained(gather_batch, ggrid, 256, 0, w->st, dx, dt, d_order + size_t(k) * batch, img * LB_WS_IN,
-                                img * LB_WS_OUT, w->act[0], bt);
-            s = loss_grad(w, bt, batch, H, Wd, d_loss + k);
+            e = lbk::launch_chained(gather_batch, ggrid, 256, 0, w->st, dx, dt, d_order + size_t(k) * batch,
+                                    img * LB_WS_IN, img * LB_WS_OUT, w->act[0], bt);
+            s = e == cudaSuccess ? loss_grad(w, bt, batch, H, Wd, d_loss + k) : launch_failed(e);
             if (s != LB_OK) break;   // no optimiser step without a gradient
             ++w->adam_t;
             const float c1 = 1.f - std::pow(b1, float(w->adam_t)), c2 = 1.f - std::pow(b2, float(w->adam_t));
-            lbk::launch_chained(adam_pack, 128, 256, 0, w->st, w->p, w->p16, w->g, w->m, w->v, w->nparams, lr, b1, b2, eps,
-                                c1, c2);
+            e = lbk::launch_chained(adam_pack, 128, 256, 0, w->st, w->p, w->p16, w->g, w->m, w->v, w->nparams, lr, b1, b2,
+                                    eps, c1, c2);
+            if (e != cudaSuccess) s = launch_failed(e);
         }
         if (s != LB_OK) break;
         e = cudaMemcpyAsync(losses.data(), d_loss, size_t(nb) * sizeof(double), cudaMemcpyDeviceToHost, w->st);

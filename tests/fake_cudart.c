@@ -10,7 +10,7 @@ enum { SUCCESS = 0, INVALID_VALUE = 1, NO_MEMORY = 2, INVALID_CONFIG = 9, NO_DEV
 
 /* ---- what the tests set and read */
 static long long capacity = -1, used = 0;      /* bytes of device memory, -1: unlimited */
-static char fail_kernel[128] = "";             /* launches of kernels whose name holds this are refused */
+static char fail_kernel[128] = "";             /* one launch of a kernel whose name holds this is refused */
 static int fail_after = 0;                     /* ... after so many that are not */
 static int no_device = 0;
 static int last_error = SUCCESS;
@@ -51,7 +51,10 @@ void __cudaRegisterFunction(void** h, const char* host, char* dev, const char* n
 static int launch(const void* fn) {
     for (int k = 0; k < nkernels; ++k)
         if (kernels[k].fn == fn) {
-            if (fail_kernel[0] && strstr(kernels[k].name, fail_kernel) && fail_after-- <= 0) return done(INVALID_CONFIG);
+            if (fail_kernel[0] && strstr(kernels[k].name, fail_kernel) && fail_after-- <= 0) {
+                fail_kernel[0] = 0;
+                return done(INVALID_CONFIG);
+            }
             ++kernels[k].launches;
             return SUCCESS;
         }
