@@ -543,9 +543,11 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
     const int elem0 = p->storage == LB_F64 ? 8 : 4;
     const int elemi = p->storage == LB_F64 ? 8 : (p->storage == LB_F32 ? 4 : 2);
     c->buf_bytes = c->pitch * (elem0 + size_t(c->Q - 1) * elemi);
+    // without a usable device the allocations below fail; until then the dispatch rules divide by sms
     int dev = 0, sms = 0, occ = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(sms, 1);
     c->ks = c->D == 2 ? lbk_kernels_d2q9(p->scheme, p->storage, p->nx, p->ny, sms)
                       : lbk_kernels_d3q19(p->scheme, p->storage, p->nx, p->ny, p->nz);
     if (!c->ks.step) { delete c; return fail(LB_EINVAL, "no kernel for this combination"); }
