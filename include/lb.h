@@ -114,7 +114,8 @@ lb_status lb_coexistence(double a, double b, double T, double* rho_l, double* rh
  * D3Q19 float64 contexts also allocate a workspace of 11 (forcing scheme) or 1
  * float64 per site, at most 1 GiB, and D3Q19 forcing contexts of 32-bit arithmetic
  * whose step takes its densities from a field one float32 per site; where these
- * cannot be had they step without them.
+ * cannot be had they step without them, and they give them back and go on without
+ * them when another allocation of the context fails.
  * LB_EINVAL also for more than 2^31 - 1 sites (the kernels index sites with
  * 32-bit integers). */
 lb_status lb_create(const lb_params* p, void* cuda_stream, lb_ctx** out);
@@ -128,7 +129,8 @@ lb_status lb_population_bytes(const lb_params* p, size_t* bytes);
  * pointer on the current device, 256-byte aligned, with at least
  * lb_population_bytes(p) bytes; it is used as is (no copy), must outlive the
  * context and is not freed by lb_destroy.  Both are checked on the host
- * before any device work (LB_EINVAL).  Everything else as lb_create. */
+ * before any device work (LB_EINVAL).  Everything else as lb_create: the status
+ * word, the work list and the workspaces named there are the context's own. */
 lb_status lb_create_with_buffers(const lb_params* p, void* cuda_stream, void* populations, size_t bytes,
                                  lb_ctx** out);
 

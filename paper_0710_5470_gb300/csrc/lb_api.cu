@@ -116,6 +116,8 @@ struct lb_ctx {
     cudaStream_t stream = nullptr;
     unsigned* d_status = nullptr;
     LbKernelSet ks;
+    LbKernelSet ks_fused;     // the form that needs neither rho32 nor work64
+    int sms = 1;
     int lz = 1;
     dim3 grid;
     int4* d_work = nullptr;   // 3D: per-CTA (x0, y0, z0, z1)
@@ -244,6 +246,72 @@ std::vector<int4> build_work_list(long long sms, long long occ, int nx, int ny, 
     return work;
 }
 
+// Launch geometry of c->ks, and for D3Q19 its work list: one CTA per TX x TY column tile and z
+// chunk; the z chunk is sized so that all CTAs are resident at once where possible.
+lb_status plan_step(lb_ctx* c) {
+    const lb_params* p = &c->p;
+    if (c->work64) {
+        c->grid = dim3(unsigned((size_t(p->nx) * p->ny * std::min(c->lz, p->nz) + c->ks.threads - 1) / c->ks.threads));
+        return LB_OK;
+    }
+    int occ = 1;
+    cudaFuncSetAttribute(c->ks.step_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(c->ks.smem));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, c->ks.step_fn, c->ks.threads, c->ks.smem) !=
+            cudaSuccess || occ < 1)
+        occ = 1;
+    cudaGetLastError();
+    const int gx = (p->nx + c->ks.tx - 1) / c->ks.tx;
+    const int gy = (p->ny + c->ks.ty - 1) / c->ks.ty;
+    c->lz = 1;
+    c->grid = dim3(gx, gy, 1);
+    if (c->ks.march_warps > 0) {
+        c->lz = c->ks.ty;
+        c->grid = dim3(unsigned(((long long)gx * gy + c->ks.march_warps - 1) / c->ks.march_warps), 1, 1);
+    }
+    if (c->D == 3) {
+        const std::vector<int4> work = build_work_list(c->sms, occ, p->nx, p->ny, p->nz, c->ks.tx, c->ks.ty);
+        c->lz = work.front().w - work.front().z;
+        cudaFree(c->d_work);
+        c->d_work = nullptr;
+        if (cudaMalloc(&c->d_work, work.size() * sizeof(int4)) != cudaSuccess ||
+            cudaMemcpy(c->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(LB_ENOMEM, "work list");
+        }
+        c->grid = dim3(unsigned(work.size()), 1, 1);
+    }
+    return LB_OK;
+}
+
+// Gives the step's workspace back and goes on with the fused form (the layout of the
+// populations is the same): what it saves in time is not worth a call that fails for want
+// of memory.  False: there is none.
+bool release_workspace(lb_ctx* c) {
+    if (!c->rho32 && !c->work64) return false;
+    cudaGetLastError();                 // of the allocation that failed
+    cudaStreamSynchronize(c->stream);   // steps in flight use it
+    for (cudaGraphExec_t& g : c->step_graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+    cudaFree(c->rho32);
+    cudaFree(c->work64);
+    c->rho32 = nullptr;
+    c->work64 = nullptr;
+    c->ks = c->ks_fused;
+    if (plan_step(c) != LB_OK) c->sticky = LB_ENOMEM;
+    return c->sticky == LB_OK;
+}
+
+// cudaMalloc for a call of the context.
+template <class T>
+cudaError_t device_alloc(lb_ctx* c, T** ptr, size_t bytes) {
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e == cudaErrorMemoryAllocation && release_workspace(c)) e = cudaMalloc(ptr, bytes);
+    if (e != cudaSuccess) cudaGetLastError();   // reported by the caller, not left for the next launch
+    return e;
+}
+
 constexpr int GRAPH_STEPS = 64;
 
 // Captures GRAPH_STEPS launches of launch_one, starting from buffer c->cur, into
@@ -272,7 +340,7 @@ cudaError_t capture_steps(lb_ctx* c, F& launch_one, cudaGraphExec_t* exec) {
 // The density staging array alone (the initialisation paths need no more).
 lb_status ensure_rho(lb_ctx* c) {
     if (c->w_rho) return LB_OK;
-    cudaError_t e = cudaMalloc(&c->w_rho, c->N * sizeof(double));
+    cudaError_t e = device_alloc(c, &c->w_rho, c->N * sizeof(double));
     if (e != cudaSuccess) {
         c->w_rho = nullptr;
         return fail(LB_ENOMEM, std::string("density array: ") + cudaGetErrorString(e));
@@ -290,10 +358,10 @@ lb_status ensure_work(lb_ctx* c) {
     c->stat_blocks = int(std::min<size_t>(1024, (n + lbk::FR_THREADS - 1) / lbk::FR_THREADS));
     if (c->stat_blocks < 1) c->stat_blocks = 1;
     cudaError_t e = cudaSuccess;
-    if ((!c->w_u && (e = cudaMalloc(&c->w_u, 3 * n * sizeof(double))) != cudaSuccess) ||
-        (!c->w_v && (e = cudaMalloc(&c->w_v, 3 * n * sizeof(double))) != cudaSuccess) ||
-        (!c->w_mp && (e = cudaMalloc(&c->w_mp, nmc * n * sizeof(double))) != cudaSuccess) ||
-        (e = cudaMalloc(&c->w_part, (size_t(c->stat_blocks) + 1) * lbk::FR_NQ * sizeof(double))) != cudaSuccess) {
+    if ((!c->w_u && (e = device_alloc(c, &c->w_u, 3 * n * sizeof(double))) != cudaSuccess) ||
+        (!c->w_v && (e = device_alloc(c, &c->w_v, 3 * n * sizeof(double))) != cudaSuccess) ||
+        (!c->w_mp && (e = device_alloc(c, &c->w_mp, nmc * n * sizeof(double))) != cudaSuccess) ||
+        (e = device_alloc(c, &c->w_part, (size_t(c->stat_blocks) + 1) * lbk::FR_NQ * sizeof(double))) != cudaSuccess) {
         c->w_part = nullptr;
         return fail(LB_ENOMEM, std::string("work arrays: ") + cudaGetErrorString(e));
     }
@@ -302,7 +370,7 @@ lb_status ensure_work(lb_ctx* c) {
 
 lb_status ensure_io(lb_ctx* c) {
     if (c->w_io) return LB_OK;
-    cudaError_t e = cudaMalloc(&c->w_io, size_t(c->Q) * c->N * sizeof(double));
+    cudaError_t e = device_alloc(c, &c->w_io, size_t(c->Q) * c->N * sizeof(double));
     if (e != cudaSuccess) return fail(LB_ENOMEM, std::string("staging buffer: ") + cudaGetErrorString(e));
     return LB_OK;
 }
@@ -544,10 +612,10 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
     const int elemi = p->storage == LB_F64 ? 8 : (p->storage == LB_F32 ? 4 : 2);
     c->buf_bytes = c->pitch * (elem0 + size_t(c->Q - 1) * elemi);
     // without a usable device the allocations below fail; until then the dispatch rules divide by sms
-    int dev = 0, sms = 0, occ = 1;
+    int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    sms = std::max(sms, 1);
+    c->sms = sms = std::max(sms, 1);
     c->ks = c->D == 2 ? lbk_kernels_d2q9(p->scheme, p->storage, p->nx, p->ny, sms)
                       : lbk_kernels_d3q19(p->scheme, p->storage, p->nx, p->ny, p->nz);
     if (!c->ks.step) { delete c; return fail(LB_EINVAL, "no kernel for this combination"); }
@@ -582,8 +650,10 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
     }
     cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream);
 
-    // D3Q19 forcing scheme in 32 bits: in two passes where that is faster and a density
-    // field is to be had, else the fused kernel (the layout of the populations is the same)
+    // D3Q19 in passes where that is faster and their workspace is to be had, else the fused
+    // kernel (the layout of the populations is the same): forcing scheme in 32 bits with a
+    // density field, and float64
+    c->ks_fused = c->ks;
     if (c->D == 3 && p->scheme == LB_SCHEME_FORCING && p->storage != LB_F64 && !std::getenv("LB_D3_VARIANT") &&
         !std::getenv("LB_NO_PAIR") && lbk_fd_wanted(p->storage, p->nx, c->N)) {
         if (cudaMalloc(&c->rho32, c->pitch * sizeof(float)) == cudaSuccess) {
@@ -593,45 +663,21 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
             cudaGetLastError();
         }
     }
-    // launch geometry of the fused step: one CTA per TX x TY column tile and z chunk;
-    // the z chunk is sized so that all CTAs are resident at once where possible.
-    cudaFuncSetAttribute(c->ks.step_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(c->ks.smem));
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, c->ks.step_fn, c->ks.threads, c->ks.smem) !=
-            cudaSuccess || occ < 1)
-        occ = 1;
-    cudaGetLastError();
-    // float64 D3Q19: in passes where their workspace is to be had, else the fused kernel
     if (c->D == 3 && p->storage == LB_F64) {
-        size_t bytes = 0;
-        const int slab = lbk_f64_slab(p->scheme, p->nx, p->ny, p->nz, &bytes);
-        if (slab > 0 && cudaMalloc(&c->work64, bytes) == cudaSuccess) {
+        size_t ws = 0;
+        const int slab = lbk_f64_slab(p->scheme, p->nx, p->ny, p->nz, &ws);
+        if (slab > 0 && cudaMalloc(&c->work64, ws) == cudaSuccess) {
             c->ks = lbk_f64_passes(p->scheme, c->ks);
             c->lz = slab;
-            c->grid = dim3(unsigned((size_t(p->nx) * p->ny * std::min(slab, p->nz) + c->ks.threads - 1) / c->ks.threads));
         } else {
             c->work64 = nullptr;
             cudaGetLastError();
         }
     }
-    if (!c->work64) {
-        const int gx = (p->nx + c->ks.tx - 1) / c->ks.tx;
-        const int gy = (p->ny + c->ks.ty - 1) / c->ks.ty;
-        c->lz = 1;
-        c->grid = dim3(gx, gy, 1);
-        if (c->ks.march_warps > 0) {
-            c->lz = c->ks.ty;
-            c->grid = dim3(unsigned(((long long)gx * gy + c->ks.march_warps - 1) / c->ks.march_warps), 1, 1);
-        }
-        if (c->D == 3) {
-            const std::vector<int4> work = build_work_list(sms, occ, p->nx, p->ny, p->nz, c->ks.tx, c->ks.ty);
-            c->lz = work.front().w - work.front().z;
-            if (cudaMalloc(&c->d_work, work.size() * sizeof(int4)) != cudaSuccess ||
-                cudaMemcpy(c->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess) {
-                lb_destroy(c);
-                return fail(LB_ENOMEM, "work list");
-            }
-            c->grid = dim3(unsigned(work.size()), 1, 1);
-        }
+    s = plan_step(c);
+    if (s != LB_OK && !release_workspace(c)) {
+        lb_destroy(c);
+        return s;
     }
     c->probe_in[0] = p->nx / 2;
     c->probe_in[1] = p->ny / 2;
@@ -758,7 +804,7 @@ lb_status lb_init_drops(lb_ctx* c, int ndrops, const double* centres, const doub
     const size_t nd = size_t(ndrops) * (c->D + 1);
     cudaError_t e = cudaSuccess;
     if (ndrops > 0) {
-        e = cudaMalloc(&d_drops, nd * sizeof(double));
+        e = device_alloc(c, &d_drops, nd * sizeof(double));
         if (e != cudaSuccess) return fail(LB_ENOMEM, "drop list");
         std::vector<double> h(nd);
         std::memcpy(h.data(), centres, size_t(ndrops) * c->D * sizeof(double));
@@ -852,7 +898,7 @@ lb_status lb_get_populations_box(lb_ctx* c, int x0, int y0, int z0, int bx, int 
     if (!c->initialised) return fail(LB_ESTATE, "state not initialised");
     double* d = nullptr;
     const size_t bytes = size_t(c->Q) * n * sizeof(double);
-    cudaError_t e = cudaMalloc(&d, bytes);
+    cudaError_t e = device_alloc(c, &d, bytes);
     if (e != cudaSuccess) return fail(LB_ENOMEM, std::string("box staging: ") + cudaGetErrorString(e));
     const int o[3] = {x0, y0, z0}, b[3] = {bx, by, bz};
     e = c->ks.get_box(pop_ptrs(c, c->cur), grid3(c), o, b, d, c->stream);
@@ -975,7 +1021,7 @@ lb_status lb_stats_get(lb_ctx* c, lb_stats* out) {
     if ((s = compute_fields(c, true, true)) != LB_OK) return s;
     const size_t du = size_t(c->D) * c->N;
     if (!c->w_uprev) {
-        cudaError_t e = cudaMalloc(&c->w_uprev, du * sizeof(double));
+        cudaError_t e = device_alloc(c, &c->w_uprev, du * sizeof(double));
         if (e != cudaSuccess) {
             c->w_uprev = nullptr;
             return fail(LB_ENOMEM, std::string("previous velocity field: ") + cudaGetErrorString(e));
