@@ -82,10 +82,15 @@ LbKernelSet pick(int storage, LbKernelSet k) {
 // per SM on, where a wave of a dozen rows and more fills the chip, tiles -> strips, chained
 // launches: 1100^2 13.8 -> 12.5, 1200 x 1100 14.6 -> 13.3, 700 x 2000 15.7 -> 14.1, 3000 x 400
 // 13.4 -> 12.4, 1500 x 1400 22.4 -> 18.6; 1024^2 (6,900 per SM) 11.8 -> 12.4, 800^2 8.1 -> 9.5.
+// Not where the strips overhang the lattice by a fifth more than tiles of 32 columns do; at
+// 4.2e6 sites, by the columns and the ratio of the overhangs: 62 (1.88) 43.4 -> 65.6, 64 (1.88) 41.7
+// -> 63.3, 128 (1.41) 43.3 -> 49.0, 192 (1.25) 44.0 -> 44.0, 96 (1.25) 42.6 -> 44.1, 250 (1.17)
+// 46.0 -> 42.7, 160 (1.13) 43.5 -> 40.5, 120 (0.94) 46.2 -> 36.8.
 int march_rows(int nx, int ny, int sms) {
     if (const char* e = std::getenv("LB_D2_ROWS")) return std::min(ny, std::max(0, std::atoi(e)));
     if (nx % 2 != 0 || double(nx) * ny < 7.2e3 * sms) return 0;
     const long long strips = (nx + MARCH_COLS - 1) / MARCH_COLS;
+    if (double(strips * MARCH_COLS) > 1.2 * 32.0 * ((nx + 31) / 32)) return 0;
     int best = 0;
     double cost = 0;
     for (int r = 12; r <= 64 && r <= ny; ++r) {
