@@ -812,12 +812,19 @@ lb_status compute_fields(lb_binary* c, bool need_u, bool need_v, bool need_mu) {
 bool is_fin(double v) { return std::isfinite(v); }
 
 // Whether a float32 D3Q19 lattice runs the marching step (LB_B3_MARCH=0 / 1 forces
-// it, for comparisons).  Small lattices give its long CTAs too little to share out:
-// us per step, bricks / march, 32^3 6.8 / 13.2 (forcing) and 4.8 / 10.2 (equilibrium),
-// 48^3 15.3 / 14.9 and 10.9 / 11.5, 64^3 24.3 / 19.7 and 17.2 / 15.7.
-bool march3_wanted(long long sites) {
+// it, for comparisons): from 2.55e5 sites of its bricks (32 x 4 x 2, overhang included) on.
+// Smaller lattices give its long CTAs too little to share out: us per step, bricks /
+// march, 32^3 6.8 / 13.2 (forcing) and 4.8 / 10.2 (equilibrium), 48^3 15.3 / 14.8 and 10.9 /
+// 12.0, 54^3 18.6 / 21.2 and 13.4 / 16.3, 60^3 (2.3e5) 21.1 / 20.4 and 15.0 / 16.4, 62^3 (2.54e5)
+// 25.1 / 23.3 and 18.4 / 18.3, 64^3 (2.62e5) 24.4 / 19.9 and 17.4 / 15.9, 48 x 64 x 64 (2.62e5)
+// 23.6 / 19.1 and 16.3 / 15.3, 33 x 70 x 70 (3.2e5) 27.4 / 24.4 and 18.0 / 19.3.  Rows of a tile that
+// lie beyond the lattice cost the equilibrium scheme more than bricks do, where fewer than
+// half lie in it: 512 x 1 x 512 31.7 / 35.5, 512 x 3 x 200 20.7 / 22.3 (forcing 56.8 / 54.0 and
+// 30.6 / 30.8), 256 x 4 x 256 17.0 / 16.7.
+bool march3_wanted(bool forcing, int nx, int ny, int nz) {
     if (const char* e = std::getenv("LB_B3_MARCH")) return std::atoi(e) != 0;
-    return sites >= 150000;
+    const auto pad = [](int n, int t) { return double((n + t - 1) / t) * t; };
+    return pad(nx, 32) * pad(ny, 4) * pad(nz, 2) >= 2.55e5 && (forcing || ny >= 4);
 }
 
 }  // namespace
@@ -866,7 +873,7 @@ lb_status lb_binary_create(const lb_binary_params* p, void* stream, lb_binary** 
     c->stream = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMalloc(&c->pop, 2 * c->set_bytes);
     if (e == cudaSuccess && c->D == 3) e = cudaMalloc(&c->phi, size_t(c->N) * c->esize);
-    if (e == cudaSuccess && c->D == 3 && p->storage == LB_F32 && march3_wanted(c->N)) {
+    if (e == cudaSuccess && c->D == 3 && p->storage == LB_F32 && march3_wanted(p->scheme == LB_SCHEME_FORCING, p->nx, p->ny, p->nz)) {
         int dev = 0, sms = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
