@@ -85,12 +85,18 @@ LbKernelSet pick(int storage, LbKernelSet k) {
 // Not where the strips overhang the lattice by a fifth more than tiles of 32 columns do; at
 // 4.2e6 sites, by the columns and the ratio of the overhangs: 62 (1.88) 43.4 -> 65.6, 64 (1.88) 41.7
 // -> 63.3, 128 (1.41) 43.3 -> 49.0, 192 (1.25) 44.0 -> 44.0, 96 (1.25) 42.6 -> 44.1, 250 (1.17)
-// 46.0 -> 42.7, 160 (1.13) 43.5 -> 40.5, 120 (0.94) 46.2 -> 36.8.
+// 46.0 -> 42.7, 160 (1.13) 43.5 -> 40.5, 120 (0.94) 46.2 -> 36.8.  Nor where the least time of the
+// strips (0.184 us a unit below 2e6 sites) is above what tiles take, 0.75 us and 1.55 ns for each
+// site of theirs per SM: 40000 x 30 13.7 -> 14.7, 80000 x 15 13.8 -> 14.7; 100000 x 12 15.8 -> 12.3,
+// 60000 x 20 14.7 -> 14.4, 20000 x 64 13.9 -> 13.1.  Tiles have no launch for more than 65535 of
+// their rows: such a lattice keeps the strips.
 int march_rows(int nx, int ny, int sms) {
     if (const char* e = std::getenv("LB_D2_ROWS")) return std::min(ny, std::max(0, std::atoi(e)));
     if (nx % 2 != 0 || double(nx) * ny < 7.2e3 * sms) return 0;
     const long long strips = (nx + MARCH_COLS - 1) / MARCH_COLS;
-    if (double(strips * MARCH_COLS) > 1.2 * 32.0 * ((nx + 31) / 32)) return 0;
+    const double tile_x = 32.0 * ((nx + 31) / 32), tile_y = 8.0 * ((ny + 7) / 8);
+    const bool tiles = tile_y <= 8.0 * 65535;
+    if (tiles && double(strips * MARCH_COLS) > 1.2 * tile_x) return 0;
     int best = 0;
     double cost = 0;
     for (int r = 12; r <= 64 && r <= ny; ++r) {
@@ -101,7 +107,7 @@ int march_rows(int nx, int ny, int sms) {
             cost = c;
         }
     }
-    return best;
+    return tiles && 0.184 * cost > 0.75 + 1.55e-3 * tile_x * tile_y / sms ? 0 : best;
 }
 
 // The pair kernel for D2Q9 with 32-bit arithmetic (storage 1, 2, 3) in place
