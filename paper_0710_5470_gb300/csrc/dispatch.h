@@ -34,14 +34,9 @@ struct LbKernelSet {
     cudaError_t (*set_pops)(const lbk::PopPtrs&, size_t n, const double* in, cudaStream_t) = nullptr;
 };
 
-// scheme: 0 equilibrium, 1 forcing; storage: lb_storage value.
-// Whether pair kernels may take tiles of 64 x ty sites in place of 32 x 8: not where
-// their overhang over the lattice is a fifth larger (LB_WIDE=0 / 1 forces it, for
-// comparisons).  A warp of a 64-wide tile stores whole rows: a row pushed one site
-// aside touches one more sector per 64 sites instead of one per 32.
-bool lbk_wide(int nx, int ny, int ty);
+// scheme: 0 equilibrium, 1 forcing; storage: lb_storage value; sms: SMs of the device.
 LbKernelSet lbk_kernels_d2q9(int scheme, int storage, int nx, int ny, int sms);
-LbKernelSet lbk_kernels_d3q19(int scheme, int storage, int nx, int ny, int nz);
+LbKernelSet lbk_kernels_d3q19(int scheme, int storage, int nx, int ny, int nz, int sms);
 
 // The float64 D3Q19 step in passes (kern_d3q19_f64.cu): planes per slab and bytes
 // of its workspace (0: no slab of a useful depth fits the workspace's limit; the

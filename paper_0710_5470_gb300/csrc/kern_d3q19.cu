@@ -15,12 +15,12 @@ static LbKernelSet pick(int storage) {
 }
 
 LbKernelSet lbk_pk_forcing(int storage, int nx, LbKernelSet base);       // kern_d3q19_pk.cu
-LbKernelSet lbk_pk_equilibrium(int storage, int nx, int ny, int nz, LbKernelSet base);   // kern_d3q19_pk_eq.cu
+LbKernelSet lbk_pk_equilibrium(int storage, int nx, int ny, int nz, int sms, LbKernelSet base);   // kern_d3q19_pk_eq.cu
 
-LbKernelSet lbk_kernels_d3q19(int scheme, int storage, int nx, int ny, int nz) {
+LbKernelSet lbk_kernels_d3q19(int scheme, int storage, int nx, int ny, int nz, int sms) {
     if (scheme != 1) {
         LbKernelSet k = pick<false>(storage);
-        return storage == 0 ? k : lbk_pk_equilibrium(storage, nx, ny, nz, k);
+        return storage == 0 ? k : lbk_pk_equilibrium(storage, nx, ny, nz, sms, k);
     }
     LbKernelSet k = pick<true>(storage);
     return storage == 0 ? k : lbk_pk_forcing(storage, nx, k);

@@ -617,7 +617,7 @@ lb_status create_impl(const lb_params* p, void* cuda_stream, void* pop_buf, size
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     c->sms = sms = std::max(sms, 1);
     c->ks = c->D == 2 ? lbk_kernels_d2q9(p->scheme, p->storage, p->nx, p->ny, sms)
-                      : lbk_kernels_d3q19(p->scheme, p->storage, p->nx, p->ny, p->nz);
+                      : lbk_kernels_d3q19(p->scheme, p->storage, p->nx, p->ny, p->nz, sms);
     if (!c->ks.step) { delete c; return fail(LB_EINVAL, "no kernel for this combination"); }
     // two sites per halo load need an even nx; LB_NO_PAIR selects the
     // one-site form (same arithmetic) everywhere, for comparison
