@@ -23,6 +23,7 @@
 #include "binary_common.cuh"
 #include "binary_launch.h"
 #include "chain.cuh"
+#include "step_kernel.cuh"   // lbk::tree_sum
 
 namespace lbb {
 
@@ -35,13 +36,24 @@ constexpr int BX = 32, BY = 4;
 template <class real>
 constexpr int brick_z() { return 2; }
 
-template <class real>
+// TREE (marching step): the populations 1.. in a balanced tree.  phi enters every equilibrium
+// population, and summed one after the other it was most of the step's rounding error: g against
+// float64 (2-norm) after 1 and 100 steps of a drop at tau = tau_phi = 1 was 1.5e-7 and 0.8e-7 off
+// (bricks 0.9e-7 and 0.9e-7), with the tree 0.3e-7 and 0.4e-7.
+template <class real, bool TREE>
 __global__ void binary_phi_kernel(const real* src, unsigned pitch, unsigned n, real* phi) {
     lbk::chain_begin();
     for (unsigned s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         real p = 0;
+        if constexpr (TREE) {
+            real g[Q3];
 #pragma unroll
-        for (int i = 0; i < Q3; ++i) p += src[(Q3 + i) * pitch + s];
+            for (int i = 0; i < Q3; ++i) g[i] = src[(Q3 + i) * pitch + s];
+            p = g[0] + lbk::tree_sum<1, Q3>(g);
+        } else {
+#pragma unroll
+            for (int i = 0; i < Q3; ++i) p += src[(Q3 + i) * pitch + s];
+        }
         phi[s] = p;
     }
 }
@@ -334,7 +346,8 @@ cudaError_t step3_impl(const StepArgs<real>& a, real* phi_buf, cudaStream_t st, 
         attr = true;
     }
     const unsigned n = unsigned(a.nx) * unsigned(a.ny) * unsigned(a.nz);
-    const cudaError_t e = lbk::launch_chained(binary_phi_kernel<real>, blocks3(n), 256, 0, st, a.src, a.pitch, n, phi_buf);
+    const cudaError_t e = lbk::launch_chained(work ? binary_phi_kernel<real, sizeof(real) == 4> : binary_phi_kernel<real, false>,
+                                              blocks3(n), 256, 0, st, a.src, a.pitch, n, phi_buf);
     if (e != cudaSuccess) return e;
     StepArgs<real> b = a;
     b.phi = phi_buf;
