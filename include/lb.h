@@ -226,13 +226,18 @@ lb_status lb_set_state(lb_ctx* ctx, const void* buf, size_t bytes);
  *
  * A library built with -DLB_DEBUG_BOUNDS (paper_0710_5470_gb300.build,
  * debug=True: _build_debug/liblb_debug.so) tests the site index of every
- * global population access of the fused step kernels against the lattice
- * before making it; an out-of-range access is skipped and the first one is
- * recorded (no trap).  lb_debug_bounds returns whether this library has the
- * checks (*checked = 1) and the first recorded violation since the last call
- * (*violation: 0 if none, else bit 63 set, the kind of access in bits 48..55 -
- * 1/2/3 pair-kernel load/store/shared write, 4/5 D3Q19 tile load/store, 6/7
- * D2Q9 load/store - and the site index in bits 0..47), then clears it.
+ * global population access of the liquid-gas step kernels (single lattices and
+ * batches, every form) and of the binary D3Q19 marching step against the
+ * lattice, and the accesses of the steps in passes to their density field and
+ * workspace against those, before making them; an out-of-range access is
+ * skipped and the first one is recorded (no trap).  The other binary kernels
+ * and the diagnostics have no checks.  lb_debug_bounds returns whether this
+ * library has the checks (*checked = 1) and the first recorded violation since
+ * the last call (*violation: 0 if none, else bit 63 set, the kind of access in
+ * bits 48..55 - 1/2/3 pair-kernel load/store/shared write, 4/5 D3Q19 one-site
+ * load/store, 6/7/8 D2Q9 load/store/shared write, 9 density field or
+ * workspace, 10/11 binary march load/store - and the index in bits 0..47),
+ * then clears it.
  * Synchronises the device.  Either pointer may be NULL. */
 lb_status lb_debug_bounds(int* checked, unsigned long long* violation);
 

@@ -32,3 +32,6 @@ cudaError_t binary_march3(bool forcing, const StepArgs<float>& a, const int4* wo
 }
 
 }  // namespace lbb
+
+// First recorded index violation of this unit's kernels (checked builds; see bounds.cuh).
+LB_BOUNDS_READER(lbk_bounds_b3march)

@@ -28,6 +28,8 @@
 namespace lbb {
 
 using lbk::fma;
+using lbk::BK_B3_LOAD;
+using lbk::BK_B3_STORE;
 
 struct March3Args {
     StepArgs<float> s;
@@ -202,6 +204,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, 3) binary_step_kernel3_march(co
         for (int m = 0; m < NA; ++m) {
             if (tid + m * NTH < NIT) {
                 const unsigned q = ld_off + a_in[m];
+                LB_GUARD(q + W - 1 < vol, BK_B3_LOAD, q, rn[m] = make_float2(0.f, 0.f); continue)
                 if constexpr (AL) rn[m] = reinterpret_cast<const float2*>(a.phi)[q >> 1];
                 else rn[m].x = a.phi[q];
             }
@@ -212,6 +215,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, 3) binary_step_kernel3_march(co
     // population k (f_0..f_18, g_0..g_18) of the own pair of the plane collided next
     auto load = [&](int k) -> P2 {
         const unsigned q = unsigned(k) * pitch + zr[1] + yr[1];
+        LB_GUARD(zr[1] + yr[1] + xc < vol && zr[1] + yr[1] + xp1 < vol, BK_B3_LOAD, zr[1] + yr[1] + xc, return pp(0.f))
         if constexpr (AL) return P2{reinterpret_cast<const float2*>(src)[(q + xc) >> 1]};
         else return pp(src[q + xc], src[q + xp1]);
     };
@@ -291,6 +295,8 @@ __global__ void __launch_bounds__((TX / 2) * TY, 3) binary_step_kernel3_march(co
                 constexpr int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
                 const unsigned row = unsigned(set + i) * pitch + zr[1 + ez] + yr[1 + ey];
                 const unsigned xa = ex == 0 ? xc : (ex == 1 ? xp1 : xm1), xb = ex == 0 ? xp1 : (ex == 1 ? xp2 : xc);
+                LB_GUARD(zr[1 + ez] + yr[1 + ey] + xa < vol && zr[1 + ez] + yr[1 + ey] + xb < vol, BK_B3_STORE,
+                         zr[1 + ez] + yr[1 + ey] + xa, return)
                 if constexpr (AL && ex == 0) {
                     reinterpret_cast<float2*>(dst)[(row + xc) >> 1] = v.v;
                 } else {

@@ -22,6 +22,9 @@ enum BoundsKind : unsigned {
     BK_2D_LOAD = 6,     // D2Q9 tile (single lattice and batch) loads
     BK_2D_STORE = 7,    // D2Q9 tile push stores
     BK_2D_SHARED = 8,   // D2Q9 pair kernel: M' shared-memory writes
+    BK_WORK = 9,        // density field and workspace of the D3Q19 steps in passes
+    BK_B3_LOAD = 10,    // binary D3Q19 marching step: phi and population loads
+    BK_B3_STORE = 11,   // binary D3Q19 marching step: push stores
 };
 
 #ifdef LB_DEBUG_BOUNDS

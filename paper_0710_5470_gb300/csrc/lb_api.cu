@@ -516,6 +516,7 @@ unsigned long long lbk_bounds_d3pke();
 unsigned long long lbk_bounds_batch();
 unsigned long long lbk_bounds_d3f64();
 unsigned long long lbk_bounds_d3fd();
+unsigned long long lbk_bounds_b3march();
 
 extern "C" {
 
@@ -1091,7 +1092,7 @@ lb_status lb_debug_bounds(int* checked, unsigned long long* violation) {
     if (checked) *checked = lbk::kBoundsChecked ? 1 : 0;
     unsigned long long v = 0;
     for (unsigned long long w : {lbk_bounds_d3pk(), lbk_bounds_d3pke(), lbk_bounds_d3q19(), lbk_bounds_d2q9(), lbk_bounds_d2pk(),
-                                 lbk_bounds_batch(), lbk_bounds_d3f64(), lbk_bounds_d3fd()})
+                                 lbk_bounds_batch(), lbk_bounds_d3f64(), lbk_bounds_d3fd(), lbk_bounds_b3march()})
         if (!v) v = w;
     if (violation) *violation = v;
     return LB_OK;

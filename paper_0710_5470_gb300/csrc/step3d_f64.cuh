@@ -94,6 +94,13 @@ __device__ __forceinline__ bool site3(const Args64x3& a, Site3& s) {
     return true;
 }
 
+// Whether the workspace planes lo..hi beside the site's lie in the workspace (checked builds).
+__device__ __forceinline__ bool planes_inside(const Args64x3& a, const Site3& s, int lo, int hi) {
+    for (int d = lo; d <= hi; ++d)
+        if ((long long)s.wp[1 + d] + (long long)a.nx * a.ny > a.field) return false;
+    return true;
+}
+
 // Sum of the 19 populations in pairs of opposite velocities.
 __device__ __forceinline__ double density19_f64(const double (&f)[19]) {
     return f[0] + tree_sum<1, 19>(f);
@@ -104,6 +111,8 @@ __global__ void __launch_bounds__(THREADS64) density3_f64(const Args64x3 a) {
     Site3 s;
     if (!site3(a, s)) return;
     const size_t q = (size_t(s.z) * a.ny + s.y) * a.nx + s.x;
+    LB_GUARD(q < size_t(a.nx) * a.ny * a.nz, BK_3D_LOAD, q, return)
+    LB_GUARD(planes_inside(a, s, 0, 0), BK_WORK, s.wp[1], return)
     double f[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) f[i] = a.src[i * a.pitch + q];
@@ -141,6 +150,7 @@ __global__ void __launch_bounds__(THREADS64) mprime3_f64(const Args64x3 a) {
     Site3 s;
     if (!site3(a, s)) return;
     const unsigned at = s.at(0, 0, 0);
+    LB_GUARD(planes_inside(a, s, -1, 1), BK_WORK, at, return)
     double g[3], lap;
     stencil19_f64(a.rho, s, a.rho[at], g, lap);
 #pragma unroll
@@ -321,6 +331,8 @@ __global__ void __launch_bounds__(THREADS64, 16) collide3_f64(const Args64x3 a) 
     const unsigned lp[3] = {unsigned(s.z == 0 ? a.nz - 1 : s.z - 1) * area, unsigned(s.z) * area,
                             unsigned(s.z == a.nz - 1 ? 0 : s.z + 1) * area};
     const unsigned q = lp[1] + s.row[1] + s.col[1];
+    LB_GUARD(q < area * unsigned(a.nz), BK_3D_LOAD, q, return)
+    LB_GUARD(planes_inside(a, s, -1, 1), BK_WORK, at, return)
     double f[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) f[i] = a.src[i * a.pitch + q];

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(256) density_pairs(const StepArgs a, unsigned 
     const unsigned t = blockIdx.x * 256u + threadIdx.x;
     if (t >= pairs) return;
     const unsigned q = 2u * t;
+    LB_GUARD((long long)q + 1 < a.pitch, BK_WORK, q, return)
     const float2 f0 = reinterpret_cast<const float2*>(a.src_base)[t];
     typename IO::W w[18];
     if constexpr (AOS) {
@@ -145,7 +146,7 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
         for (int m = 0; m < NA; ++m) {
             if (tid + m * NTH < NIT) {
                 const unsigned q = unsigned(ld_off) + a_in[m];
-                LB_GUARD(size_t(q) + 1 < nsites, BK_PK_LOAD, q, rn[m] = make_float2(0.f, 0.f); continue)
+                LB_GUARD(size_t(q) + 1 < nsites, BK_WORK, q, rn[m] = make_float2(0.f, 0.f); continue)
                 rn[m] = reinterpret_cast<const float2*>(field)[q >> 1];
             }
         }
@@ -273,8 +274,8 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) step_kernel3d_fd(const St
                 auto store = [&](auto I, P2 v) {
                     constexpr int i = decltype(I)::value;
                     constexpr int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
-                    const unsigned row = unsigned(zr[1 + ez]) + yr[1 + ey];
-                    const unsigned xa = ex == 0 ? xc : (ex == 1 ? xp1 : xm1), xb = ex == 0 ? xp1 : (ex == 1 ? xp2 : xc);
+                    [[maybe_unused]] const unsigned row = unsigned(zr[1 + ez]) + yr[1 + ey];
+                    [[maybe_unused]] const unsigned xa = ex == 0 ? xc : (ex == 1 ? xp1 : xm1), xb = ex == 0 ? xp1 : (ex == 1 ? xp2 : xc);
                     LB_GUARD(size_t(row) + xa < nsites && size_t(row) + xb < nsites, BK_PK_STORE, row + xa, return)
                     if constexpr (AOS) {
                         char* b = args.dst[1] + zb[1 + ez] + yb[1 + ey] + (i - 1) * ROWB;
@@ -394,7 +395,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) step_kernel3d_fd1(const StepArgs
         for (int m = 0; m < NA; ++m) {
             if (tid + m * NT < RN) {
                 const unsigned q = unsigned(ld_off + a_in[m]);
-                LB_GUARD(q < unsigned(vol), BK_3D_LOAD, q, rn[m] = 0.f; continue)
+                LB_GUARD(q < unsigned(vol), BK_WORK, q, rn[m] = 0.f; continue)
                 rn[m] = args.rho32[q];
             }
         }
