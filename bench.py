@@ -34,35 +34,37 @@ WORKLOAD = dict(lattice="D3Q19", n=128, R=30.0, scheme="forcing", T=0.55, kappa=
 BYTES_POP = {"f64": (8, 8), "f32": (4, 4), "f16dev": (4, 2), "bf16dev": (4, 2)}   # (f_0, f_i) bytes
 
 
-KERNEL_SOURCES = ["step3d.cuh", "step3d_pk.cuh", "kern_d3q19_pk.cu", "step_kernel.cuh", "storage.cuh", "lattice.cuh"]
-# DRAM bytes (read + write) per launch of the D3Q19 forcing step kernel at
+KERNEL_SOURCES = ["step3d.cuh", "step3d_pk.cuh", "kern_d3q19_pk.cu", "step3d_fd.cuh", "kern_d3q19_fd.cu",
+                  "step3d_f64.cuh", "kern_d3q19_f64.cu", "step_kernel.cuh", "storage.cuh", "lattice.cuh"]
+# DRAM bytes (read + write) per step (all its kernels) of the D3Q19 forcing scheme at
 # 128^3, from ncu (dram__bytes_read.sum + dram__bytes_write.sum), keyed by the
 # fingerprint of the kernel sources they were measured on and the storage.
 # A changed kernel has a new fingerprint and reports traffic = null.
 NCU_TRAFFIC = {
-    ("412489fce235", "f16dev", 128): 142.85e6,   # 103.35 MB read + 39.50 MB written (pair kernel)
-    ("412489fce235", "bf16dev", 128): 143.09e6,  # 103.39 MB read + 39.70 MB written (pair kernel)
-    ("412489fce235", "f32", 128): 301.60e6,      # 188.75 MB read + 112.85 MB written (pair kernel, 2 CTAs per SM)
-    ("412489fce235", "f64", 128): 637.11e6,      # 357.07 MB read + 280.05 MB written (tile kernel)
+    ("a5152197534b", "f16dev", 128): 220.4e6,    # density pass 83.9 MB read, 2.6 written; step 94.4 and 39.5
+    ("a5152197534b", "bf16dev", 128): 219.8e6,   # 83.9 and 2.7; 94.4 and 38.8
+    ("a5152197534b", "f32", 128): 444.6e6,       # 159.4 and 5.0; 170.3 and 109.9
+    ("a5152197534b", "f64", 128): 1244.4e6,      # density 318.8 and 14.9; M' 17.1 and 105.4; collision 505.2 and 283.0
 }
 
-# Executed floating-point operations per lattice update of the step kernel,
-# from ncu's per-opcode instruction counts of one launch divided by the sites
+# Executed floating-point operations per lattice update of the step's kernels,
+# from ncu's per-opcode instruction counts of one step divided by the sites
 # (FFMA, DFMA, FADD2, FMUL2 = 2 flops, FFMA2 = 4; FADD, FMUL, FHADD, DADD,
 # DMUL = 1), keyed like
 # NCU_TRAFFIC.  They include the halo recomputation, so they are the work the
 # FP units do, not an algorithmic minimum.
 NCU_FLOPS = {
-    # pair kernel: FFMA 10.8, FADD 64.3, FMUL 20.6, FADD2 36.6, FFMA2 43.9, FMUL2 29.9, FHADD 75.2 per site
-    ("412489fce235", "f16dev", 128): 490.5,
-    # float32 pair kernel: FFMA 10.3, FADD 61.5, FMUL 17.8, FADD2 64.8, FFMA2 43.5, FMUL2 29.6
-    ("412489fce235", "f32", 128): 462.7,
-    ("412489fce235", "f64", 128): 525.6,       # tile kernel: DFMA 129.0, DADD 197.4, DMUL 70.2
+    # density pass: FHADD 18, FADD2 1 per site; step: FFMA 10.8, FADD 64.3, FMUL 20.6, FADD2 34.2, FFMA2 43.9,
+    # FMUL2 29.9, FHADD 30.0
+    ("a5152197534b", "f16dev", 128): 460.3,
+    ("a5152197534b", "bf16dev", 128): 460.3,
+    ("a5152197534b", "f32", 128): 450.3,     # FADD2 9.5; FFMA 10.8, FADD 64.3, FMUL 20.6, FADD2 44.7, FFMA2 43.9, FMUL2 29.9
+    ("a5152197534b", "f64", 128): 406.0,     # DADD 18; DADD 34, DFMA 10, DMUL 8; DADD 110, DFMA 95, DMUL 26
 }
 # FP64-pipe instructions per lattice update of the float64 step (DFMA, DADD,
-# DMUL, DSETP, F2F): each occupies the pipe like one FMA, so their rate against
+# DMUL, DSETP): each occupies the pipe like one FMA, so their rate against
 # half the FMA flop rate is the pipe's utilisation.
-NCU_FP64_PIPE_OPS = {("412489fce235", "f64", 128): 401.7}
+NCU_FP64_PIPE_OPS = {("a5152197534b", "f64", 128): 303.0}
 
 
 def alu_roofline(fp: str, storage: str, n: int, glups: float, fma: dict | None):
@@ -102,12 +104,19 @@ def bytes_per_lu(storage: str, q: int = 19) -> int:
     return 2 * (b0 + (q - 1) * bi) + 2 * s_rho
 
 
-def bytes_moved_per_lu(storage: str, q: int = 19) -> int:
-    """Bytes per lattice update this design moves: the populations once in and
-    once out (the density is recomputed on chip and never stored): 80 B for
-    16-bit deviations, 152 B float32, 304 B float64."""
+def bytes_moved_per_lu(storage: str, q: int = 19, form: str = "") -> int:
+    """Bytes per lattice update that a step of this form (lb_kernel_info) moves, every value that
+    a kernel reads or writes counted once per kernel.  Fused: the populations in and out, 80 B for
+    16-bit deviations, 152 B float32, 304 B float64.  With a density field: the populations once
+    more and the field written and read, 128 B and 236 B.  Float64 in two passes the same, 472 B;
+    in three passes also the gradient, Laplacian and six M' fields, 640 B."""
     b0, bi = BYTES_POP[storage]
-    return 2 * (b0 + (q - 1) * bi)
+    pops = b0 + (q - 1) * bi
+    if "density field" in form or "two passes" in form:
+        return 3 * pops + 2 * (8 if storage == "f64" else 4)
+    if "three passes" in form:
+        return 3 * pops + 8 * (1 + 1 + 10 + 1 + 10)
+    return 2 * pops
 
 
 def parse():
@@ -548,12 +557,13 @@ def run_native(args):
     st = ctx.stats()
     ms, mlups = whole_job(dist, world, sites, args.steps, ms_local)
 
-    # roofline of the fused step kernel (the only kernel in the timed region):
-    # algorithmic bytes per launch / average launch duration
+    # roofline of the step (its kernels are the only ones in the timed region):
+    # algorithmic bytes per step / average duration of a step
     bpl = bytes_per_lu(args.storage)
+    moved = bytes_moved_per_lu(args.storage, form=kinfo["form"])
     t_launch = ms_local / args.steps / 1e3
     achieved = bpl * sites / t_launch / 1e9
-    # the ncu tables hold the forcing-scheme kernel
+    # the ncu tables hold the forcing scheme
     forcing = args.scheme == "forcing"
     traffic = NCU_TRAFFIC.get((fp, args.storage, n)) if forcing else None
     # FMA rates of this GPU (float64 and float32), best of three short launches
@@ -686,8 +696,7 @@ def run_native(args):
                        "parallelism": f"{world} independent replica(s)"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "bytes_per_lu": bpl,
-                         "bytes_moved_per_lu": bytes_moved_per_lu(args.storage),
-                         "frac_of_moved": achieved * bytes_moved_per_lu(args.storage) / bpl / peak,
+                         "bytes_moved_per_lu": moved, "frac_of_moved": achieved * moved / bpl / peak,
                          "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback",
                          "kernel_fingerprint": fp},
             "alu_roofline": alu,

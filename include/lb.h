@@ -174,11 +174,12 @@ lb_status lb_get_populations(lb_ctx* ctx, double* f);
 #define LB_BOX_MAX_LOG2_SITES 24
 lb_status lb_get_populations_box(lb_ctx* ctx, int x0, int y0, int z0, int bx, int by, int bz, double* f);
 
-/* Advance nsteps >= 0 time steps of Eq. 4: one fused kernel per step
- * (moments, stencils, equilibrium, force, BGK, streaming).  Asynchronous on
+/* Advance nsteps >= 0 time steps of Eq. 4 (moments, stencils, equilibrium,
+ * force, BGK, streaming): one fused kernel per step, or two or three where the
+ * context steps in passes (lb_kernel_info).  Asynchronous on
  * the context's stream; a non-finite density raises the context's status,
  * reported by the next synchronising call.  With nsteps > 64 the steps run
- * as replays of a CUDA graph of 64 kernel launches (captured once per
+ * as replays of a CUDA graph of 64 steps (captured once per
  * starting buffer on a private stream of the context, after one ordinary
  * launch) plus ordinary launches for the rest; the results are identical. */
 lb_status lb_step(lb_ctx* ctx, int nsteps);
@@ -276,11 +277,13 @@ lb_status lb_shape(const lb_ctx* ctx, long long* n_sites, int* q);
  * rows of 32 values of a block contiguous, 1152 bytes; site q in block q/32). */
 lb_status lb_device_state(lb_ctx* ctx, void** dptr, size_t* bytes);
 
-/* Launch form of the context's fused step kernel (Eq. 4 per site, one launch
- * per time step): a short description written into name (at most cap bytes,
- * NUL-terminated; name may be NULL), the CTA's column tile (tile_x x tile_y
- * sites), threads per CTA, dynamic shared memory per CTA, and the number of
- * CTAs per launch.  Any output pointer may be NULL. */
+/* Launch form of the context's step (Eq. 4 per site): a short description
+ * written into name (at most cap bytes, NUL-terminated; name may be NULL), the
+ * CTA's column tile (tile_x x tile_y sites), threads per CTA, dynamic shared
+ * memory per CTA and CTAs per launch of the kernel that collides and streams.
+ * One launch per time step, but two where the description says "density field"
+ * or "two passes" and three for "three passes" (per slab of planes where the
+ * lattice exceeds the workspace).  Any output pointer may be NULL. */
 lb_status lb_kernel_info(const lb_ctx* ctx, char* name, size_t cap, int* tile_x, int* tile_y, int* threads,
                          size_t* smem, int* ctas);
 
