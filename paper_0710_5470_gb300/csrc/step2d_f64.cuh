@@ -81,11 +81,10 @@ __device__ __forceinline__ void collide9_f64(const double (&f)[9], double rho, d
     const double jx = a1 + (a5 - a7), jy = a3 + (a5 + a7);
     const double ob = fma(-k.b, rho, 1.0);
     const double r = 1.0 / (rho * ob);
-    const double irho = r * ob, ib0 = r * rho;
-    // 1 / (1 - b rho) to half a unit (one Newton step): p0 multiplies its error several times (collide19_f64)
-    const double ib = fma(ib0, fma(-ob, ib0, 1.0), ib0);
+    const double irho = r * ob, ib = r * rho;
     const double ux = jx * irho, uy = jy * irho;
-    const double Tib = k.T * ib;
+    // T / (1 - b rho) to half a unit (one Newton step): p0 multiplies its error several times (collide19_f64)
+    const double Tib0 = k.T * ib, Tib = fma(ib, fma(-ob, Tib0, k.T), Tib0);
     const double p0 = rho * fma(-k.a, rho, Tib);                                      // Eq. 2
     const double lam12 = fma(-k.nu12x3, Tib * ib, fma(k.nu12x6a, rho, k.nu12));       // Eq. 36, over 12
     const double lx = lam12 * ux, ly = lam12 * uy;

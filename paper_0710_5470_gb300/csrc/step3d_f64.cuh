@@ -236,12 +236,11 @@ __device__ __forceinline__ void collide19_f64(const double (&f)[19], double rho,
     }
     const double ob = fma(-k.b, rho, 1.0);
     const double r = 1.0 / (rho * ob);
-    const double irho = r * ob, ib0 = r * rho;
-    // 1 / (1 - b rho) to half a unit: p0 is a small difference of T ib and a rho, which multiplies the error
-    // of ib several times (one Newton step, two operations; without it the populations' error against
+    const double irho = r * ob, ib = r * rho;
+    // T / (1 - b rho) to half a unit: p0 is a small difference of it and a rho, which multiplies its
+    // error several times (one Newton step, two operations; without it the populations' error against
     // exact arithmetic was 7 - 17% larger, 20 steps of a drop)
-    const double ib = fma(ib0, fma(-ob, ib0, 1.0), ib0);
-    const double Tib = k.T * ib;
+    const double Tib0 = k.T * ib, Tib = fma(ib, fma(-ob, Tib0, k.T), Tib0);
     const double p0 = rho * fma(-k.a, rho, Tib);                                     // Eq. 2
     const double olam = fma(-k.onu12x3, Tib * ib, fma(k.onu12x6a, rho, k.onu12));    // omega lambda/12, Eq. 36
     // omega Q_ab + u_a g_b + u_b g_a = omega j_a u_b + u_a w_b + u_b w_a + delta_ab omega lambda u.G
