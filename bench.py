@@ -41,10 +41,10 @@ KERNEL_SOURCES = ["step3d.cuh", "step3d_pk.cuh", "kern_d3q19_pk.cu", "step3d_fd.
 # fingerprint of the kernel sources they were measured on and the storage.
 # A changed kernel has a new fingerprint and reports traffic = null.
 NCU_TRAFFIC = {
-    ("a5152197534b", "f16dev", 128): 220.4e6,    # density pass 83.9 MB read, 2.6 written; step 94.4 and 39.5
-    ("a5152197534b", "bf16dev", 128): 219.8e6,   # 83.9 and 2.7; 94.4 and 38.8
-    ("a5152197534b", "f32", 128): 444.6e6,       # 159.4 and 5.0; 170.3 and 109.9
-    ("a5152197534b", "f64", 128): 1244.4e6,      # density 318.8 and 14.9; M' 17.1 and 105.4; collision 505.2 and 283.0
+    ("a45ef727e828", "f16dev", 128): 220.4e6,    # density pass 83.9 MB read, 2.6 written; step 94.4 and 39.5
+    ("a45ef727e828", "bf16dev", 128): 219.8e6,   # 83.9 and 2.7; 94.4 and 38.8
+    ("a45ef727e828", "f32", 128): 444.6e6,       # 159.4 and 5.0; 170.3 and 109.9
+    ("a45ef727e828", "f64", 128): 1244.4e6,      # density 318.8 and 14.9; M' 17.1 and 105.4; collision 505.2 and 283.0
 }
 
 # Executed floating-point operations per lattice update of the step's kernels,
@@ -56,15 +56,15 @@ NCU_TRAFFIC = {
 NCU_FLOPS = {
     # density pass: FHADD 18, FADD2 1 per site; step: FFMA 10.8, FADD 64.3, FMUL 20.6, FADD2 34.2, FFMA2 43.9,
     # FMUL2 29.9, FHADD 30.0
-    ("a5152197534b", "f16dev", 128): 460.3,
-    ("a5152197534b", "bf16dev", 128): 460.3,
-    ("a5152197534b", "f32", 128): 450.3,     # FADD2 9.5; FFMA 10.8, FADD 64.3, FMUL 20.6, FADD2 44.7, FFMA2 43.9, FMUL2 29.9
-    ("a5152197534b", "f64", 128): 406.0,     # DADD 18; DADD 34, DFMA 10, DMUL 8; DADD 110, DFMA 95, DMUL 26
+    ("a45ef727e828", "f16dev", 128): 460.3,
+    ("a45ef727e828", "bf16dev", 128): 460.3,
+    ("a45ef727e828", "f32", 128): 450.3,     # FADD2 9.5; FFMA 10.8, FADD 64.3, FMUL 20.6, FADD2 44.7, FFMA2 43.9, FMUL2 29.9
+    ("a45ef727e828", "f64", 128): 406.0,     # DADD 18; DADD 34, DFMA 10, DMUL 8; DADD 110, DFMA 95, DMUL 26
 }
 # FP64-pipe instructions per lattice update of the float64 step (DFMA, DADD,
 # DMUL, DSETP): each occupies the pipe like one FMA, so their rate against
 # half the FMA flop rate is the pipe's utilisation.
-NCU_FP64_PIPE_OPS = {("a5152197534b", "f64", 128): 303.0}
+NCU_FP64_PIPE_OPS = {("a45ef727e828", "f64", 128): 303.0}
 
 
 def alu_roofline(fp: str, storage: str, n: int, glups: float, fma: dict | None):
