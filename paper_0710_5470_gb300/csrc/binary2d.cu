@@ -878,15 +878,17 @@ lb_status lb_binary_create(const lb_binary_params* p, void* stream, lb_binary** 
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int occ = binary_march3_ctas(p->scheme == LB_SCHEME_FORCING, p->nx);
-        lb_work_list(sms, occ, p->nx, p->ny, p->nz, 32, 8, nullptr, 0, &c->ctas);
         std::vector<int4> work;
+        if (lb_work_list(sms, occ, p->nx, p->ny, p->nz, 32, 8, nullptr, 0, &c->ctas) != LB_OK) e = cudaErrorMemoryAllocation;
         try {
             work.resize(size_t(c->ctas));
         } catch (...) {
             e = cudaErrorMemoryAllocation;
         }
+        if (e == cudaSuccess &&
+            lb_work_list(sms, occ, p->nx, p->ny, p->nz, 32, 8, reinterpret_cast<int*>(work.data()), c->ctas, &c->ctas) != LB_OK)
+            e = cudaErrorMemoryAllocation;
         if (e == cudaSuccess) {
-            lb_work_list(sms, occ, p->nx, p->ny, p->nz, 32, 8, reinterpret_cast<int*>(work.data()), c->ctas, &c->ctas);
             e = cudaMalloc(&c->d_work, work.size() * sizeof(int4));
         }
         if (e == cudaSuccess)

@@ -44,7 +44,12 @@ struct PKELaunch {
 double waves(int sms, int occ, double c0, int nx, int ny, int nz, int tx, int ty) {
     int n = 0;
     if (lb_work_list(sms, occ, nx, ny, nz, tx, ty, nullptr, 0, &n) != LB_OK) return 0.0;
-    std::vector<int> list(4 * size_t(n));
+    std::vector<int> list;
+    try {
+        list.resize(4 * size_t(n));
+    } catch (...) {
+        return 0.0;
+    }
     lb_work_list(sms, occ, nx, ny, nz, tx, ty, list.data(), n, &n);
     double t = 0.0;
     for (long long k = 0; k < n; k += (long long)sms * occ) {

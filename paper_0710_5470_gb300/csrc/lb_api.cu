@@ -269,7 +269,12 @@ lb_status plan_step(lb_ctx* c) {
         c->grid = dim3(unsigned(((long long)gx * gy + c->ks.march_warps - 1) / c->ks.march_warps), 1, 1);
     }
     if (c->D == 3) {
-        const std::vector<int4> work = build_work_list(c->sms, occ, p->nx, p->ny, p->nz, c->ks.tx, c->ks.ty);
+        std::vector<int4> work;
+        try {
+            work = build_work_list(c->sms, occ, p->nx, p->ny, p->nz, c->ks.tx, c->ks.ty);
+        } catch (...) {
+            return fail(LB_ENOMEM, "work list on the host");
+        }
         c->lz = work.front().w - work.front().z;
         cudaFree(c->d_work);
         c->d_work = nullptr;
@@ -873,7 +878,12 @@ lb_status lb_work_list(int sms, int ctas_per_sm, int nx, int ny, int nz, int til
     if (sms < 1 || ctas_per_sm < 1 || nx < 1 || ny < 1 || nz < 1 || tile_x < 1 || tile_y < 1 ||
         (long long)nx * ny * nz > 0x7fffffffLL)
         return fail(LB_EINVAL, "sizes must be positive (at most 2^31 - 1 sites)");
-    const std::vector<int4> w = build_work_list(sms, ctas_per_sm, nx, ny, nz, tile_x, tile_y);
+    std::vector<int4> w;
+    try {
+        w = build_work_list(sms, ctas_per_sm, nx, ny, nz, tile_x, tile_y);
+    } catch (...) {
+        return fail(LB_ENOMEM, "work list on the host");
+    }
     if (w.size() > size_t(0x7fffffff)) return fail(LB_EINVAL, "work list too long");
     *count = int(w.size());
     if (out)

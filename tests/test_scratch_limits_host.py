@@ -40,3 +40,19 @@ fake.fake_capacity(fake.fake_used() + 1000)
 print(json.dumps([status(c.fields), status(c.step, 3), status(c.synchronize)]))
 """, tmp_path)
     assert out == [2, 0, 0]
+
+
+@pytest.mark.parametrize("scheme,storage,nx", [(0, 2, 34), (0, 1, 37), (1, 2, 37), (1, 0, 2)])
+def test_a_work_list_beyond_the_hosts_memory_is_an_error_code(scheme, storage, nx, tmp_path):
+    """A lattice of hundreds of millions of column tiles under a limit of the process's memory: LB_ENOMEM, no
+    exception through the C entry."""
+    out = fakecuda.run(f"""
+import resource
+lb.load_library()
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + 400_000_000,) * 2)
+st = status(lb.Context, 1, ({nx}, {2_000_000_000 // nx}, 1), A_VDW, B_VDW, 0.55, 0.01, 0.8, {scheme}, {storage}, buffer=(1 << 20, 1 << 50))
+one = status(lb.work_list, 152, 2, ({nx}, {2_000_000_000 // nx}, 1), (1, 1))
+print(json.dumps([st, one]))
+""", tmp_path)
+    assert out == [2, 2]
