@@ -115,7 +115,8 @@ lb_status lb_coexistence(double a, double b, double T, double* rho_l, double* rh
  * float64 per site, at most 1 GiB, and D3Q19 forcing contexts of 32-bit arithmetic
  * whose step takes its densities from a field one float32 per site; where these
  * cannot be had they step without them, and they give them back and go on without
- * them when another allocation of the context fails.
+ * them when another allocation of the context fails (float64 results then
+ * differ in their last place, all others not at all).
  * LB_EINVAL also for more than 2^31 - 1 sites (the kernels index sites with
  * 32-bit integers). */
 lb_status lb_create(const lb_params* p, void* cuda_stream, lb_ctx** out);
